@@ -313,6 +313,48 @@ int device_sms() {
   return nsm;
 }
 
+// Scratch of the path through operand images (attend_dense.cu): the heads are
+// taken in `groups` equal groups, each with its images and the partial results
+// of its split query blocks.
+constexpr size_t kDenseImages = (size_t)1 << 40;   // images of one group, at most (one head at least)
+
+struct DenseGroups {
+  int heads;        // of a group (the last may have fewer)
+  size_t images;    // bytes
+  size_t bytes;     // the whole scratch
+};
+
+DenseGroups dense_groups(int64_t Nq, int H, int64_t Nk, int nsm) {
+  const size_t head = qwm::dense_head_bytes(qwm::plan_dense(Nq, 1, Nk, nsm));
+  const int64_t most = (int64_t)(kDenseImages / head);
+  const int n = most < 1 ? H : (int)((H + most - 1) / most);
+  DenseGroups g{};
+  g.heads = (H + n - 1) / n;
+  g.images = (size_t)g.heads * head;
+  const int last = H - (H - 1) / g.heads * g.heads;
+  const size_t p0 = qwm::dense_part_bytes(qwm::plan_dense(Nq, g.heads, Nk, nsm));
+  const size_t p1 = qwm::dense_part_bytes(qwm::plan_dense(Nq, last, Nk, nsm));
+  g.bytes = g.images + (p0 > p1 ? p0 : p1);
+  return g;
+}
+
+// Every cached token and the active ones; *units: cached chunks and the active
+// chunk, *longest: the tokens of the longest of them.
+int64_t total_keys(const qwm_cache* c, int64_t N_cur, int* units, int64_t* longest) {
+  const int32_t n = qwm_cache_num_chunks(c);
+  int64_t keys = N_cur, most = N_cur;
+  for (int32_t i = 0; i < n; ++i) {
+    int64_t tok;
+    int32_t s;
+    qwm_cache_chunk_info(c, i, &s, &tok);
+    keys += tok;
+    most = tok > most ? tok : most;
+  }
+  *units = n + (N_cur > 0 ? 1 : 0);
+  *longest = most;
+  return keys;
+}
+
 qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q, int64_t Nq, const void* k_cur,
                        const void* v_cur, int64_t N_cur, float sm_scale, void* out, float* lse, void* workspace,
                        size_t workspace_bytes, void* stream) {
@@ -338,6 +380,51 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
     slots.tokens[i] = (int32_t)tok;
     slots.psac[i] = c->psac[s];
   }
+  const int nsm = device_sms();
+  if (nsm <= 0) return QWM_ERR_CUDA;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+
+  int units = 0;
+  int64_t longest = 0;
+  const int64_t Nk = total_keys(c, N_cur, &units, &longest);
+  // The images' path gives no log-sum-exp: that is fp32, and its last digits
+  // follow where the running maximum and the binary16 probabilities are
+  // rounded, which the other kernel's results fix.  The idle role of the
+  // timeout test belongs to that kernel too.
+  if (workspace && units >= 2 && !lse && c->idle_role == 0) {
+    const DenseGroups g = dense_groups(Nq, c->L.H, Nk, nsm);
+    if (workspace_bytes >= g.bytes) {
+      qwm::DenseArgs d{};
+      d.L = c->L;
+      d.base = c->base;
+      d.status = reinterpret_cast<int32_t*>(c->base);
+      d.q = static_cast<const __nv_bfloat16*>(q);
+      d.kcur = static_cast<const __nv_bfloat16*>(k_cur);
+      d.vcur = static_cast<const __nv_bfloat16*>(v_cur);
+      d.Nq = Nq;
+      d.Ncur = N_cur;
+      d.Nk = Nk;
+      d.sm_scale = sm_scale;
+      d.out = static_cast<__nv_bfloat16*>(out);
+      d.wait_ns = c->wait_ns;
+      d.img = static_cast<uint8_t*>(workspace);
+      d.part_o = reinterpret_cast<float*>(d.img + g.images);
+      int64_t key = 0;
+      for (int32_t i = 0; i <= n; ++i) {
+        d.key0[i] = key;
+        if (i < n) key += slots.tokens[i];
+      }
+      for (int h0 = 0; h0 < c->L.H; h0 += g.heads) {
+        const int heads = c->L.H - h0 < g.heads ? c->L.H - h0 : g.heads;
+        const qwm::DensePlan p = qwm::plan_dense(Nq, heads, Nk, nsm);
+        d.h0 = h0;
+        d.part_ml = d.part_o + (size_t)p.tail_ctas * 2 * 256 * 128;
+        if (qwm::launch_dense(d, slots, p, heads, (int)((longest + 127) / 128), st) != cudaSuccess) return QWM_ERR_CUDA;
+      }
+      return QWM_OK;
+    }
+  }
+
   qwm::AttendArgs a{};
   a.L = c->L;
   a.base = c->base;
@@ -352,11 +439,9 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
   a.lse = lse;
   a.wait_ns = c->wait_ns;
   a.idle_role = c->idle_role;
-  const int nsm = device_sms();
-  if (nsm <= 0) return QWM_ERR_CUDA;
-  qwm::AttendPlan pl = qwm::plan_attend(Nq, c->L.H, n + (N_cur > 0 ? 1 : 0), nsm, workspace != nullptr);
+  qwm::AttendPlan pl = qwm::plan_attend(Nq, c->L.H, units, nsm, workspace != nullptr);
   const size_t need = qwm::attend_workspace_bytes(pl);
-  if (need > 0 && workspace_bytes < need) pl = qwm::plan_attend(Nq, c->L.H, n + (N_cur > 0 ? 1 : 0), nsm, false);
+  if (need > 0 && workspace_bytes < need) pl = qwm::plan_attend(Nq, c->L.H, units, nsm, false);
   a.bph = pl.bph;
   a.n_units = pl.n_units;
   a.n_whole = pl.n_whole;
@@ -365,7 +450,7 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
     a.part_o = static_cast<float*>(workspace);
     a.part_ml = a.part_o + (size_t)(pl.n_units - pl.n_whole) * pl.nparts * 512 * 128;
   }
-  return qwm::launch_attend(a, slots, static_cast<cudaStream_t>(stream)) == cudaSuccess ? QWM_OK : QWM_ERR_CUDA;
+  return qwm::launch_attend(a, slots, st) == cudaSuccess ? QWM_OK : QWM_ERR_CUDA;
 }
 
 }  // namespace
@@ -379,8 +464,14 @@ size_t qwm_attend_workspace_bytes(const qwm_config* cfg, const qwm_cache* c, int
   if (!cfg || !c || Nq < 1 || N_cur < 0 || !supported(cfg) || !same_shape(cfg, &c->cfg)) return 0;
   const int nsm = device_sms();
   if (nsm <= 0) return 0;
-  const int n_key_units = qwm_cache_num_chunks(c) + (N_cur > 0 ? 1 : 0);
-  return qwm::attend_workspace_bytes(qwm::plan_attend(Nq, c->L.H, n_key_units, nsm, true));
+  int units = 0;
+  int64_t longest = 0;
+  const int64_t Nk = total_keys(c, N_cur, &units, &longest);
+  if (units < 2) return 0;
+  // enough for either path: which one runs depends on the call's lse
+  const size_t parts = qwm::attend_workspace_bytes(qwm::plan_attend(Nq, c->L.H, units, nsm, true));
+  const size_t dense = dense_groups(Nq, c->L.H, Nk, nsm).bytes;
+  return dense > parts ? dense : parts;
 }
 
 qwm_status qwm_attend_ws(const qwm_config* cfg, const qwm_cache* c, const void* q, int64_t Nq, const void* k_cur,

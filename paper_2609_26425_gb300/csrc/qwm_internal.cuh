@@ -173,6 +173,40 @@ AttendPlan plan_attend(int64_t Nq, int H, int n_key_units, int nsm, bool split);
 size_t attend_workspace_bytes(const AttendPlan& pl);
 cudaError_t launch_attend(const AttendArgs& a, const AttendSlots& slots, cudaStream_t s);
 
+// Attention through a scratch buffer (attend_dense.cu): the keys of a group of
+// heads are rebuilt once into binary16 operand images (64 KB per 128 keys and
+// head), which the attention kernel streams.
+struct DenseArgs {
+  Layout L;
+  const uint8_t* base;
+  int32_t* status;             // device status word
+  const __nv_bfloat16* q;      // [Nq][H][d]
+  const __nv_bfloat16* kcur;   // [Ncur][H][d]
+  const __nv_bfloat16* vcur;
+  int64_t Nq, Ncur, Nk;        // Nk: every cached token and the active ones
+  float sm_scale;
+  __nv_bfloat16* out;          // [Nq][H][d]
+  uint64_t wait_ns;            // limit of every bounded wait
+  int32_t h0;                  // first head of the group
+  // blocks of 256 queries of one head, numbered head by head: `waves` whole
+  // ones per CTA, then n_tail ones whose key tiles are shared out over tail_ctas
+  int32_t bph, NT, waves, n_tail, tail_ctas, tail_more;
+  int64_t tail_per;            // tail key tiles of a CTA (one more for the first tail_more)
+  uint8_t* img;                // [heads of the group][NT][K 32 KB | V 32 KB]
+  float* part_o;               // [2 tail_ctas][256][128] fp32
+  float* part_ml;              // [2 tail_ctas][256][2] fp32
+  int64_t key0[kMaxSlots + 1]; // first key of each unit (cached chunks in order, then the active chunk)
+};
+struct DensePlan {
+  int32_t bph, NT, waves, n_tail, tail_ctas, tail_more, grid, nsm;
+  int64_t tail_per;
+};
+DensePlan plan_dense(int64_t Nq, int heads, int64_t Nk, int nsm);
+size_t dense_part_bytes(const DensePlan& p);
+size_t dense_head_bytes(const DensePlan& p);   // images of one head
+cudaError_t launch_dense(const DenseArgs& a, const AttendSlots& slots, const DensePlan& p, int heads, int max_tiles,
+                         cudaStream_t st);
+
 struct FitArgs {
   int H, d, C, iters, Npad;    // Npad: C rounded up to a multiple of 16 (MMA width)
   int64_t N;
