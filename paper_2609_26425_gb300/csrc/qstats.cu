@@ -11,14 +11,10 @@
 //                 tokens of one head; the S partial sums meet in distributed
 //                 shared memory and are added to S_h in rank order, so the
 //                 result does not depend on timing.
-//   basis_kernel  w from the diagonal of S (Eq. 8) and the eigenvectors of
-//                 M = S / count by cyclic Jacobi in fp32 (Eq. 15).  A holds
-//                 its upper triangle in shared memory; each round rotates 64
-//                 disjoint index pairs (round-robin schedule) and updates each
-//                 2 x 2 block of A once, in place.  The CTAs of a cluster run
-//                 the same rotations on their own copy of A (same arithmetic,
-//                 same bits) and each accumulates its share of the rows of the
-//                 eigenvector matrix V.
+//   basis_kernel  w from the diagonal of S (Eq. 8) and the eigenvalues and
+//                 leading eigenvectors of M = S / count in fp32 (Eq. 15):
+//                 Householder tridiagonalisation, multisection, inverse
+//                 iteration, back-transformation; one CTA per head.
 #include "qwm_internal.cuh"
 #include "ptx_sm103.cuh"
 
@@ -178,40 +174,81 @@ __global__ void __launch_bounds__(kGThreads) gram_kernel(const __grid_constant__
   }
 }
 
-// ------------------------------------------------------------------ Jacobi basis
-constexpr int kJs = 129;          // padded row stride: entry (i, j) in bank (i + j) % 32
-constexpr int kJThreads = 512;
-constexpr int kMaxSweeps = 30;
+// ------------------------------------------------------------------ Query basis
+constexpr int kBThreads = 512;
+constexpr int kVecs = 32;                        // eigenvectors kept at most (the largest PSAC rank)
+constexpr int kXs = kVecs + 1;                   // row stride of the vectors [128][kXs]
+// shared memory, in floats
+constexpr int Q_HV = 0;                          // Householder vectors [126][128], unnormalised
+constexpr int Q_LU = Q_HV + 126 * 128;           // tridiagonal LU factors [4][128][kVecs]
+constexpr int Q_X = Q_LU + 4 * 128 * kVecs;      // right-hand sides, vectors [128][kXs]
+constexpr int Q_HC = Q_X + 128 * kXs;            // Householder scales [128]
+constexpr int Q_D = Q_HC + 128;                  // T: diagonal, off-diagonal, its square [128] each
+constexpr int Q_E = Q_D + 128;
+constexpr int Q_E2 = Q_E + 128;
+constexpr int Q_LAM = Q_E2 + 128;                // eigenvalues, decreasing
+constexpr int Q_XB = Q_LAM + 128;                // two buffers of 128
+constexpr int Q_RED = Q_XB + 256;                // [32]
+constexpr int Q_CNT = Q_RED + 32;                // counts at the grid points [512]
+constexpr int Q_ORD = Q_CNT + 512;               // order of a diagonal matrix [128]
+constexpr int kBasisSmem = (Q_ORD + 128) * 4;
+constexpr int kIter = 2;                         // steps of inverse iteration
+constexpr float kTinyPivot = 1.1920929e-7f;      // 2^-23 of the matrix norm
 
-__host__ __device__ constexpr int basis_smem_bytes(int vrows) {
-  return (128 + vrows) * kJs * 4   // A, V rows
-         + 4 * 64 * 4              // pair tables
-         + 32 * 4 + 128 * 4        // reductions, eigenvalue order
-         + 32 * 16 + 32 * 4;       // sign candidates, signs
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+  return x;
 }
 
-__global__ void __launch_bounds__(kJThreads, 1) basis_kernel(uint8_t* stats, float* w, __nv_bfloat16* U,
-                                                             float* evals, int r, int eig) {
-  extern __shared__ __align__(16) float js[];
-  const int SJ = (int)gridDim.x;   // CTAs of this head's cluster
-  const int rank = (int)cluster_rank();
-  const int VR = 128 / SJ;         // rows of V kept by this CTA: rank * VR + [0, VR)
-  float* A = js;                   // [128][kJs], entry (i, j) at min(i,j) * kJs + max(i,j)
-  float* V = A + 128 * kJs;        // [VR][kJs]
-  float* pc = V + VR * kJs;        // per pair: cos, sin, new a_ff, new a_gg
-  float* psn = pc + 64;
-  float* paf = psn + 64;
-  float* pag = paf + 64;
-  float* red = pag + 64;
-  int* order = reinterpret_cast<int*>(red + 32);
-  float4* cand = reinterpret_cast<float4*>(order + 128);
-  float* sgn = reinterpret_cast<float*>(cand + 32);
+// Number of eigenvalues of the tridiagonal T (norm <= 1) below x: sign changes
+// of the leading principal minors p_i = (d_i - x) p_(i-1) - e_(i-1)^2 p_(i-2).
+// A ratio p_i / p_(i-1) below 2^-26 in magnitude is taken as +2^-26 (d_i moved
+// by less than fp32's rounding of the matrix), which keeps four steps between
+// two rescalings inside the fp32 range.
+__device__ __forceinline__ int sturm_count(const float* d, const float* e2, float x) {
+  float p0 = 0.0f, p1 = 1.0f;
+  int n = 0;
+#pragma unroll 1
+  for (int i = 0; i < 128; i += 4) {
+    const float4 dv = *reinterpret_cast<const float4*>(d + i);
+    const float4 ev = *reinterpret_cast<const float4*>(e2 + i);   // e2[i] couples i - 1 and i; e2[0] = 0
+    const float dd[4] = {dv.x, dv.y, dv.z, dv.w}, ee[4] = {ev.x, ev.y, ev.z, ev.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float p = fmaf(dd[k] - x, p1, -(ee[k] * p0));
+      const float lim = 1.4901161e-8f * p1;
+      p = fabsf(p) < fabsf(lim) ? lim : p;
+      n += (int)((__float_as_uint(p) ^ __float_as_uint(p1)) >> 31);
+      p0 = p1;
+      p1 = p;
+    }
+    const float sc = __uint_as_float((254u - ((__float_as_uint(p1) >> 23) & 0xFFu)) << 23);   // 2^-exponent
+    p0 *= sc;
+    p1 *= sc;
+  }
+  return n;
+}
 
+// w from the diagonal of S (Eq. 8) and the leading eigenvectors of M = S /
+// count (Eq. 15), one CTA per head: Householder tridiagonalisation with M in
+// registers (thread = row tid / 4, a quarter of its columns), all eigenvalues
+// by multisection on Sturm counts, the r leading vectors by two steps of
+// inverse iteration from fixed pseudo-random vectors (LU with partial pivoting,
+// a thread per vector), each followed by modified Gram-Schmidt in decreasing
+// order (so equal eigenvalues get an orthonormal basis), and the Householder
+// vectors applied back (a warp per vector).  A matrix whose off-diagonal
+// entries are all below 2^-20 of its norm counts as diagonal.
+// Bound by the latency of its serial chain (126 reduction steps of two block
+// barriers, 128-step recurrences): the work is 9 n^3 operations a head.
+__global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, float* w, __nv_bfloat16* U, float* evals,
+                                                             int r, int eig) {
+  extern __shared__ __align__(16) float js[];
+  float* red = js + Q_RED;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int h = blockIdx.y;
+  const int h = blockIdx.x;
   const unsigned long long cnt = *reinterpret_cast<const unsigned long long*>(stats + 8);
   const float* S = reinterpret_cast<const float*>(stats + kStatsHeader) + (size_t)h * 128 * 128;
-  auto ut = [](int i, int j) { return i <= j ? i * kJs + j : j * kJs + i; };
 
   // ---- Eq. 8: w_c = S_cc / mean_c' S_c'c' (the 1/count of M cancels)
   if (tid < 128) {
@@ -222,205 +259,478 @@ __global__ void __launch_bounds__(kJThreads, 1) basis_kernel(uint8_t* stats, flo
     if (lane == 0) red[warp] = t;
     named_bar_sync(1, 128);
     const float sum = (red[0] + red[1]) + (red[2] + red[3]);
-    if (w && rank == 0) w[h * 128 + tid] = (cnt > 0 && sum > 0.0f) ? dg * 128.0f / sum : 1.0f;
+    if (w) w[h * 128 + tid] = (cnt > 0 && sum > 0.0f) ? dg * 128.0f / sum : 1.0f;
   }
   if (!eig) return;
   __syncthreads();
 
-  // ---- M = S / count into A (upper triangle), V = identity rows, ||M||_F
+  // ---- M = S / count: row i, columns 4 (c + 4 m) .. + 3
+  const int i = tid >> 2, c = tid & 3;
   const float inv = cnt ? (float)(1.0 / (double)cnt) : 0.0f;
-  float ss = 0.0f;
-  for (int e = tid; e < 128 * 128; e += kJThreads) {
-    const int i = e >> 7, j = e & 127;
-    const float a = S[e] * inv;
-    if (i <= j) A[i * kJs + j] = a;
-    ss = fmaf(a, a, ss);
-  }
-  for (int e = tid; e < VR * 128; e += kJThreads) {
-    const int i = e >> 7, j = e & 127;
-    V[i * kJs + j] = (rank * VR + i == j) ? 1.0f : 0.0f;
+  uint64_t a[16];
+  float top = 0.0f, offmax = 0.0f;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const float4 v = *reinterpret_cast<const float4*>(S + i * 128 + 4 * (c + 4 * m));
+    const float x[4] = {v.x * inv, v.y * inv, v.z * inv, v.w * inv};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (4 * (c + 4 * m) + e == i) js[Q_D + i] = x[e];
+      else offmax = fmaxf(offmax, fabsf(x[e]));
+      top = fmaxf(top, fabsf(x[e]));
+    }
+    a[2 * m] = f2pack(x[0], x[1]);
+    a[2 * m + 1] = f2pack(x[2], x[3]);
   }
 #pragma unroll
-  for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
+  for (int o = 16; o; o >>= 1) {
+    offmax = fmaxf(offmax, __shfl_xor_sync(0xFFFFFFFFu, offmax, o));
+    top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+  }
+  if (lane == 0) {
+    red[warp] = top;
+    red[16 + warp] = offmax;
+  }
+  __syncthreads();
+  for (int k = 0; k < 16; ++k) {
+    top = fmaxf(top, red[k]);
+    offmax = fmaxf(offmax, red[16 + k]);
+  }
+  // entries scaled (by a power of two) to at most 1
+  int ex0 = 0;
+  if (top > 0.0f && top < INFINITY) frexpf(top, &ex0);
+  ex0 = ex0 < -126 ? -126 : ex0;
+  const float sc0 = ldexpf(1.0f, -ex0);
+  float ss = 0.0f;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    float x0, x1;
+    a[m] = mul2(a[m], f2pack(sc0, sc0));
+    f2unpack(a[m], x0, x1);
+    ss = fmaf(x0, x0, fmaf(x1, x1, ss));
+  }
+  offmax *= sc0;
+  ss = warp_sum(ss);
+  __syncthreads();
   if (lane == 0) red[warp] = ss;
   __syncthreads();
   float fro2 = 0.0f;
-  for (int i = 0; i < kJThreads / 32; ++i) fro2 += red[i];
-  const float thr = ldexpf(sqrtf(fro2), -20);   // rotate pairs whose |a_fg| exceeds this
-
-  // ---- cyclic Jacobi sweeps; round rr pairs index 0 with 1 + rr and
-  // 1 + (rr + k) % 127 with 1 + (rr - k) % 127 for k = 1..63, so each sweep
-  // (127 rounds) meets every index pair once
-  auto wrap = [](int x) { return x >= 127 ? x - 127 : x; };   // x < 254
-  auto pair_f = [&](int rr, int k) { return k == 0 ? 0 : 1 + wrap(rr + k); };
-  auto pair_g = [&](int rr, int k) { return k == 0 ? 1 + rr : 1 + wrap(rr + 127 - k); };
-  int sweeps = 0;
-  for (; sweeps < kMaxSweeps; ++sweeps) {
-    int any = 0;
-#pragma unroll 1
-    for (int rr = 0; rr < 127; ++rr) {
-      int rot = 0;
-      if (tid < 64) {
-        const int f = pair_f(rr, tid), g = pair_g(rr, tid);
-        const float aff = A[f * kJs + f], agg = A[g * kJs + g], afg = A[ut(f, g)];
-        float c = 1.0f, s = 0.0f, nf = aff, ng = agg;
-        if (fabsf(afg) > thr) {
-          // the rotation that zeroes a_fg: tan = sign(tau) / (|tau| + sqrt(1 + tau^2)),
-          // |tau| <= 2^20 here; fast reciprocals: any (c, s) with c^2 + s^2 = 1
-          // to rounding is an orthogonal step, and a_fg is set to zero below
-          const float tau = __fdividef(agg - aff, 2.0f * afg);
-          const float q = fmaf(tau, tau, 1.0f);
-          const float t = __fdividef(copysignf(1.0f, tau), fabsf(tau) + q * rsqrtf(q));
-          c = rsqrtf(fmaf(t, t, 1.0f));
-          s = t * c;
-          nf = aff - t * afg;
-          ng = agg + t * afg;
-          rot = 1;
-        }
-        pc[tid] = c;
-        psn[tid] = s;
-        paf[tid] = nf;
-        pag[tid] = ng;
+  for (int k = 0; k < 16; ++k) fro2 += red[k];
+  // not above the threshold, a norm that is not finite included: diagonal
+  if (!(offmax > ldexpf(sqrtf(fro2), -20)) || !(fro2 < INFINITY)) {
+    int* order = reinterpret_cast<int*>(js + Q_ORD);
+    if (tid < 128) {   // decreasing order (equal values by increasing index; NaN last)
+      float ki = js[Q_D + tid];
+      if (ki != ki) ki = -INFINITY;
+      int rk = 0;
+      for (int j = 0; j < 128; ++j) {
+        float kj = js[Q_D + j];
+        if (kj != kj) kj = -INFINITY;
+        rk += (kj > ki) || (kj == ki && j < tid);
       }
-      if (!__syncthreads_or(rot)) continue;
-      any = 1;
-      // A <- J^T A J.  Off-diagonal 2 x 2 blocks {a, b}: warp-iteration b,
-      // lanes a = (b + 1 + lane) % 64 (lane 31 only for b < 32), so each
-      // unordered pair of pairs is updated exactly once.  The four blocks of
-      // a thread are disjoint: all loads first, then the rotations.
-      {
-        int ix[4][4];
-        float cs[4][4], x[4][4];
-        bool act[4];
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-          const int b = warp + 16 * it;
-          const int a = (b + 1 + lane) & 63;
-          cs[it][0] = pc[a];
-          cs[it][1] = psn[a];
-          cs[it][2] = pc[b];
-          cs[it][3] = psn[b];
-          act[it] = !(lane == 31 && b >= 32) && (cs[it][1] != 0.0f || cs[it][3] != 0.0f);
-          const int fa = pair_f(rr, a), ga = pair_g(rr, a), fb = pair_f(rr, b), gb = pair_g(rr, b);
-          ix[it][0] = ut(fa, fb);
-          ix[it][1] = ut(fa, gb);
-          ix[it][2] = ut(ga, fb);
-          ix[it][3] = ut(ga, gb);
-        }
-#pragma unroll
-        for (int it = 0; it < 4; ++it)
-          if (act[it])
-#pragma unroll
-            for (int e = 0; e < 4; ++e) x[it][e] = A[ix[it][e]];
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-          if (!act[it]) continue;
-          const float ca = cs[it][0], sa = cs[it][1], cb = cs[it][2], sb = cs[it][3];
-          // columns of pair b, then rows of pair a
-          const float y00 = cb * x[it][0] - sb * x[it][1], y01 = sb * x[it][0] + cb * x[it][1];
-          const float y10 = cb * x[it][2] - sb * x[it][3], y11 = sb * x[it][2] + cb * x[it][3];
-          A[ix[it][0]] = ca * y00 - sa * y10;
-          A[ix[it][2]] = sa * y00 + ca * y10;
-          A[ix[it][1]] = ca * y01 - sa * y11;
-          A[ix[it][3]] = sa * y01 + ca * y11;
-        }
-      }
-      // the diagonal block of each rotated pair in closed form
-      if (tid < 64 && psn[tid] != 0.0f) {
-        const int f = pair_f(rr, tid), g = pair_g(rr, tid);
-        A[f * kJs + f] = paf[tid];
-        A[g * kJs + g] = pag[tid];
-        A[ut(f, g)] = 0.0f;
-      }
-      // V <- V J on this CTA's rows (columns of four disjoint pairs per warp)
-      {
-        int vf[4], vg[4];
-        float vc[4], vs[4];
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-          const int b = warp + 16 * it;
-          vc[it] = pc[b];
-          vs[it] = psn[b];
-          vf[it] = pair_f(rr, b);
-          vg[it] = pair_g(rr, b);
-        }
-        for (int i = lane; i < VR; i += 32) {
-          float x[4], y[4];
-#pragma unroll
-          for (int it = 0; it < 4; ++it)
-            if (vs[it] != 0.0f) {
-              x[it] = V[i * kJs + vf[it]];
-              y[it] = V[i * kJs + vg[it]];
-            }
-#pragma unroll
-          for (int it = 0; it < 4; ++it)
-            if (vs[it] != 0.0f) {
-              V[i * kJs + vf[it]] = vc[it] * x[it] - vs[it] * y[it];
-              V[i * kJs + vg[it]] = vs[it] * x[it] + vc[it] * y[it];
-            }
-        }
-      }
-      __syncthreads();
+      order[rk] = tid;
+      if (evals) evals[h * 128 + rk] = js[Q_D + tid];
     }
-    if (!any) break;
+    if (tid == 0) atomicMax(reinterpret_cast<int*>(stats + 16), 1);
+    __syncthreads();
+    if (U)
+      for (int e = tid; e < 128 * r; e += kBThreads) {
+        const int row = e / r, j = e - row * r;
+        U[((size_t)h * 128 + row) * r + j] = __float2bfloat16_rn(cnt && order[j] == row ? 1.0f : 0.0f);
+      }
+    return;
   }
-  const int nsweeps = sweeps < kMaxSweeps ? sweeps + 1 : kMaxSweeps;
 
-  // ---- eigenvalues in decreasing order (equal values by increasing index;
-  // NaN last)
+  // ---- T = Q^T M Q: step k takes row k past the diagonal (x, zero up to k) to
+  // beta e_(k+1) with H = I - s v v^T, v = x - beta e_(k+1), s = 1 / (beta (beta
+  // - x_(k+1))); p = s A v, K = s p.v / 2, A -= v (p - K v)^T + (p - K v) v^T.
+  float* xb = js + Q_XB;
+  float* pb = xb + 128;
+  auto publish = [&](int k) {   // row k of the current matrix, by its four threads
+    if (i == k) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        float x[4];
+        f2unpack(a[2 * m], x[0], x[1]);
+        f2unpack(a[2 * m + 1], x[2], x[3]);
+        const int j0 = 4 * (c + 4 * m);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (j0 + e == k) js[Q_D + k] = x[e];
+          if (j0 + e <= k) x[e] = 0.0f;
+        }
+        *reinterpret_cast<float4*>(xb + j0) = make_float4(x[0], x[1], x[2], x[3]);
+      }
+    }
+  };
+  publish(0);
+  __syncthreads();
+#pragma unroll 1
+  for (int k = 0; k < 126; ++k) {
+    const float4 xq = reinterpret_cast<const float4*>(xb)[lane];
+    const float alpha = xb[k + 1];
+    float sig = fmaf(xq.x, xq.x, fmaf(xq.y, xq.y, fmaf(xq.z, xq.z, xq.w * xq.w)));
+    sig = warp_sum(sig);          // x_(k+1)^2 included
+    const float beta = -copysignf(sqrtf(sig), alpha);
+    const bool refl = sig > 1e-30f;   // entries are at most 1: a smaller row counts as zero
+    const float s = refl ? __fdividef(1.0f, beta * (beta - alpha)) : 0.0f;
+    const float vk1 = alpha - beta;
+    const bool live = warp * 8 + 7 > k;   // this warp still has rows past k
+    uint64_t v[16];
+    float vi = 0.0f, p = 0.0f;
+    if (live) {
+      uint64_t acc0 = 0, acc1 = 0;
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const int j0 = 4 * (c + 4 * m);
+        float4 x = *reinterpret_cast<const float4*>(xb + j0);
+        if (j0 == ((k + 1) & ~3)) {
+          const int e = (k + 1) & 3;
+          x.x = e == 0 ? vk1 : x.x;
+          x.y = e == 1 ? vk1 : x.y;
+          x.z = e == 2 ? vk1 : x.z;
+          x.w = e == 3 ? vk1 : x.w;
+        }
+        v[2 * m] = f2pack(x.x, x.y);
+        v[2 * m + 1] = f2pack(x.z, x.w);
+        acc0 = fma2(a[2 * m], v[2 * m], acc0);
+        acc1 = fma2(a[2 * m + 1], v[2 * m + 1], acc1);
+      }
+      vi = i == k + 1 ? vk1 : xb[i];
+      float y0, y1, y2, y3;
+      f2unpack(acc0, y0, y1);
+      f2unpack(acc1, y2, y3);
+      p = (y0 + y1) + (y2 + y3);
+      p += __shfl_xor_sync(0xFFFFFFFFu, p, 1);
+      p += __shfl_xor_sync(0xFFFFFFFFu, p, 2);
+      p = i > k ? p * s : 0.0f;
+      float kp = p * vi;   // the same in the four threads of a row
+      kp += __shfl_xor_sync(0xFFFFFFFFu, kp, 4);
+      kp += __shfl_xor_sync(0xFFFFFFFFu, kp, 8);
+      kp += __shfl_xor_sync(0xFFFFFFFFu, kp, 16);
+      if (lane == 0) red[warp] = kp;
+      if (c == 0) pb[i] = p;
+    } else {
+      if (lane == 0) red[warp] = 0.0f;
+      if (c == 0) pb[i] = 0.0f;
+    }
+    if (tid < 128) js[Q_HV + k * 128 + tid] = tid == k + 1 ? vk1 : xb[tid];
+    if (tid == 0) {
+      js[Q_HC + k] = s;
+      js[Q_E + k + 1] = refl ? beta : 0.0f;
+    }
+    __syncthreads();
+    if (live) {
+      float K = 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 t = reinterpret_cast<const float4*>(red)[q];
+        K += (t.x + t.y) + (t.z + t.w);
+      }
+      K *= 0.5f * s;
+      const float wi = fmaf(-K, vi, p);
+      const uint64_t nK = f2pack(-K, -K), nv = f2pack(-vi, -vi), nw = f2pack(-wi, -wi);
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const float4 q = *reinterpret_cast<const float4*>(pb + 4 * (c + 4 * m));
+        const uint64_t w0 = fma2(nK, v[2 * m], f2pack(q.x, q.y)), w1 = fma2(nK, v[2 * m + 1], f2pack(q.z, q.w));
+        a[2 * m] = fma2(nv, w0, fma2(nw, v[2 * m], a[2 * m]));
+        a[2 * m + 1] = fma2(nv, w1, fma2(nw, v[2 * m + 1], a[2 * m + 1]));
+      }
+    }
+    publish(k + 1);
+    __syncthreads();
+  }
+  if (tid == 0) {
+    js[Q_E + 127] = xb[127];   // row 126 past the diagonal
+    js[Q_E] = 0.0f;
+  }
+  __syncthreads();
+  publish(127);
+  __syncthreads();
+
+  // ---- scale T to norm <= 1 (a power of two), Gershgorin bounds
+  float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = lane + 32 * q;
+    const float rad = fabsf(js[Q_E + j]) + (j < 127 ? fabsf(js[Q_E + j + 1]) : 0.0f);
+    lo = fminf(lo, js[Q_D + j] - rad);
+    hi = fmaxf(hi, js[Q_D + j] + rad);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
+  }
+  int ex;
+  frexpf(fmaxf(fabsf(lo), fabsf(hi)), &ex);   // norm < 2^ex
+  const float scale = ldexpf(1.0f, -ex), unscale = ldexpf(1.0f, ex + ex0);
   __syncthreads();
   if (tid < 128) {
-    float ki = A[tid * kJs + tid];
-    if (ki != ki) ki = -INFINITY;
-    int rk = 0;
-    for (int j = 0; j < 128; ++j) {
-      float kj = A[j * kJs + j];
-      if (kj != kj) kj = -INFINITY;
-      rk += (kj > ki) || (kj == ki && j < tid);
+    const float e = js[Q_E + tid] * scale;
+    js[Q_D + tid] *= scale;
+    js[Q_E + tid] = e;
+    js[Q_E2 + tid] = e * e;
+  }
+  lo = lo * scale - 1e-6f;
+  hi = hi * scale + 1e-6f;
+  __syncthreads();
+
+  // ---- eigenvalues: counts at 512 points, then five-fold sections of each
+  // one's interval by a quad of threads
+  {
+    const float* d = js + Q_D;
+    const float* e2 = js + Q_E2;
+    int* gc = reinterpret_cast<int*>(js + Q_CNT);
+    const float st = (hi - lo) * (1.0f / 513.0f);
+    gc[tid] = sturm_count(d, e2, fmaf(st, (float)(tid + 1), lo));
+    __syncthreads();
+    const int idx = 127 - i;   // eigenvalue i of the decreasing order is number idx of the increasing one
+    int g0 = 0, g1 = 512;      // first grid point with more than idx eigenvalues below it
+    while (g0 < g1) {
+      const int mid = (g0 + g1) >> 1;
+      if (gc[mid] > idx) g1 = mid;
+      else g0 = mid + 1;
     }
-    order[rk] = tid;
+    float l = g0 == 0 ? lo : fmaf(st, (float)g0, lo), u = g0 == 512 ? hi : fmaf(st, (float)(g0 + 1), lo);
+#pragma unroll 1
+    for (int it = 0; it < 7; ++it) {   // 2 / 513 / 5^7 < 2^-24
+      const float wd = (u - l) * 0.2f;
+      const float x = fmaf(wd, (float)(c + 1), l);
+      const uint32_t above = __ballot_sync(0xFFFFFFFFu, sturm_count(d, e2, x) > idx) >> (lane & 28);
+      const int first = __ffs((int)((above & 15u) | 16u)) - 1;   // section of the quad that holds the eigenvalue
+      const float nl = first == 0 ? l : fmaf(wd, (float)first, l);
+      u = first == 4 ? u : fmaf(wd, (float)(first + 1), l);
+      l = nl;
+    }
+    if (c == 0) js[Q_LAM + i] = 0.5f * (l + u);
   }
   __syncthreads();
-  if (rank == 0) {
-    if (evals && tid < 128) evals[h * 128 + tid] = A[order[tid] * kJs + order[tid]];
-    if (tid == 0) atomicMax(reinterpret_cast<int*>(stats + 16), nsweeps);
+  if (warp == 0) {   // rounding may not put a value above the one before it
+    float run = INFINITY;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float x = js[Q_LAM + 32 * q + lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x = fminf(x, y);
+      }
+      x = fminf(x, run);
+      run = __shfl_sync(0xFFFFFFFFu, x, 31);
+      js[Q_LAM + 32 * q + lane] = x;
+      if (evals) evals[h * 128 + 32 * q + lane] = x * unscale;
+    }
   }
+  if (tid == 0) atomicMax(reinterpret_cast<int*>(stats + 16), kIter);
+  __syncthreads();
   if (!U || r == 0) return;
 
-  // ---- U_r: column j = eigenvector order[j], signed so that its largest
-  // |entry| (the first one on ties) is positive; the candidates of the
-  // cluster's row blocks meet through distributed shared memory
-  if (tid < r) {
-    const int col = order[tid];
-    float best = -1.0f, val = 0.0f;
-    int brow = 0;
-    for (int i = 0; i < VR; ++i) {
-      const float v = V[i * kJs + col];
-      if (fabsf(v) > best) {
-        best = fabsf(v);
-        brow = rank * VR + i;
-        val = v;
+  // ---- LU of T - lambda_j with partial pivoting (lane j of warp 0), pivots of
+  // at least 2^-23 in magnitude
+  float* fi = js + Q_LU;                 // 1 / pivot
+  float* f1 = fi + 128 * kVecs;          // first and second superdiagonal of U
+  float* f2 = f1 + 128 * kVecs;
+  float* fl = f2 + 128 * kVecs;          // multiplier
+  float* X = js + Q_X;
+  uint32_t swp[4] = {0u, 0u, 0u, 0u};    // rows swapped
+  if (warp == 0 && lane < r) {
+    const float lam = js[Q_LAM + lane];
+    float D = js[Q_D] - lam, Us = js[Q_E + 1];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll 1
+      for (int b = 0; b < 32; ++b) {
+        const int n = 32 * q + b;
+        if (n == 127) break;
+        const float e = js[Q_E + n + 1], dn = js[Q_D + n + 1] - lam, en = n < 126 ? js[Q_E + n + 2] : 0.0f;
+        float piv, m1, m2, l;
+        if (fabsf(D) >= fabsf(e)) {
+          piv = fabsf(D) < kTinyPivot ? copysignf(kTinyPivot, D) : D;
+          l = __fdividef(e, piv);
+          m1 = Us;
+          m2 = 0.0f;
+          D = fmaf(-l, Us, dn);
+          Us = en;
+        } else {
+          piv = fabsf(e) < kTinyPivot ? copysignf(kTinyPivot, e) : e;
+          l = __fdividef(D, piv);
+          m1 = dn;
+          m2 = en;
+          D = fmaf(-l, dn, Us);
+          Us = -l * en;
+          swp[q] |= 1u << b;
+        }
+        fi[n * kVecs + lane] = __fdividef(1.0f, piv);
+        f1[n * kVecs + lane] = m1;
+        f2[n * kVecs + lane] = m2;
+        fl[n * kVecs + lane] = l;
       }
     }
-    cand[tid] = make_float4(best, __int_as_float(brow), val, 0.0f);
+    if (fabsf(D) < kTinyPivot) D = copysignf(kTinyPivot, D);
+    fi[127 * kVecs + lane] = __fdividef(1.0f, D);
+    f1[127 * kVecs + lane] = 0.0f;
+    f2[127 * kVecs + lane] = 0.0f;
   }
-  cluster_sync();
-  if (tid < r) {
-    float best = -1.0f, val = 0.0f;
-    for (int src = 0; src < SJ; ++src) {
-      const float4 c = ld_dsmem_f4(mapa(smem_u32(cand + tid), (uint32_t)src));
-      if (c.x > best) {
-        best = c.x;
-        val = c.z;
+  // fixed pseudo-random start, entries of magnitude 2^-20 .. 2^-19 (a solve grows them by up to 2^23 and more)
+  for (int e = tid; e < 128 * kVecs; e += kBThreads) {
+    uint32_t z = (uint32_t)e * 2654435769u + 12345u;
+    z ^= z >> 16;
+    z *= 0x85EBCA6Bu;
+    z ^= z >> 13;
+    z *= 0xC2B2AE35u;
+    z ^= z >> 16;
+    X[(e / kVecs) * kXs + (e % kVecs)] = __uint_as_float((z & 0x807FFFFFu) | (107u << 23));
+  }
+  __syncthreads();
+  float y[2][4];   // warp wq's vectors wq and wq + 16: entries lane + 32 q
+#pragma unroll 1
+  for (int it = 0; it < kIter; ++it) {
+    if (warp == 0 && lane < r) {
+      float bc = X[lane];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t sw = swp[q];
+#pragma unroll 4
+        for (int b = 0; b < 32; ++b) {
+          const int n = 32 * q + b;
+          if (n < 127) {
+            const float nx = X[(n + 1) * kXs + lane], l = fl[n * kVecs + lane];
+            const bool s1 = (sw >> b) & 1u;
+            const float keep = s1 ? nx : bc, other = s1 ? bc : nx;
+            X[n * kXs + lane] = keep;
+            bc = fmaf(-l, keep, other);
+          }
+        }
+      }
+      float x1 = 0.0f, x2 = 0.0f;
+#pragma unroll 4
+      for (int n = 127; n >= 0; --n) {
+        const float b = n == 127 ? bc : X[n * kXs + lane];
+        const float x0 = fmaf(-f1[n * kVecs + lane], x1, fmaf(-f2[n * kVecs + lane], x2, b)) * fi[n * kVecs + lane];
+        X[n * kXs + lane] = x0;
+        x2 = x1;
+        x1 = x0;
       }
     }
-    sgn[tid] = val < 0.0f ? -1.0f : 1.0f;
+    __syncthreads();
+    // modified Gram-Schmidt, largest eigenvalue first
+#pragma unroll
+    for (int sl = 0; sl < 2; ++sl) {
+      const int j = warp + 16 * sl;
+      float mx = 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        y[sl][q] = j < r ? X[(lane + 32 * q) * kXs + j] : 0.0f;
+        mx = fmaxf(mx, fabsf(y[sl][q]));
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+      const float sc = mx > 0.0f && mx < INFINITY ? __fdividef(1.0f, mx) : 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[sl][q] = fabsf(y[sl][q]) < INFINITY ? y[sl][q] * sc : 0.0f;
+    }
+#pragma unroll 1
+    for (int j = 0; j < r; ++j) {
+      float* vb = xb + 128 * (j & 1);
+      const int own = j >> 4;
+      if (warp == (j & 15)) {
+#pragma unroll
+        for (int sl = 0; sl < 2; ++sl)
+          if (sl == own) {
+            float n2 = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) n2 = fmaf(y[sl][q], y[sl][q], n2);
+            n2 = warp_sum(n2);
+            const float sc = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              y[sl][q] *= sc;
+              vb[lane + 32 * q] = y[sl][q];
+            }
+          }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int sl = 0; sl < 2; ++sl) {
+        const int k = warp + 16 * sl;
+        if (k > j && k < r) {
+          float dt = 0.0f, b[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            b[q] = vb[lane + 32 * q];
+            dt = fmaf(b[q], y[sl][q], dt);
+          }
+          dt = warp_sum(dt);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) y[sl][q] = fmaf(-dt, b[q], y[sl][q]);
+        }
+      }
+    }
+    if (it + 1 < kIter) {
+#pragma unroll
+      for (int sl = 0; sl < 2; ++sl) {
+        const int j = warp + 16 * sl;
+        if (j < r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) X[(lane + 32 * q) * kXs + j] = y[sl][q] * 9.5367432e-7f;
+      }
+    }
+    __syncthreads();
   }
-  cluster_sync();  // candidates read by every CTA before any leaves
-  for (int e = tid; e < VR * r; e += kJThreads) {
-    const int i = e / r, j = e - i * r;
-    const float v = cnt ? sgn[j] * V[i * kJs + order[j]] : 0.0f;
-    U[((size_t)h * 128 + rank * VR + i) * r + j] = __float2bfloat16_rn(v);
+
+  // ---- back to M's coordinates: H_0 ... H_125 y; then the sign rule (the
+  // largest |entry|, the first one on ties, is positive) and bf16
+  const bool two = warp + 16 < r;
+  if (warp < r) {
+    const float* hv = js + Q_HV + 125 * 128 + lane;
+#pragma unroll 2
+    for (int k = 125; k >= 0; --k, hv -= 128) {
+      float b[4], d0 = 0.0f, d1 = 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        b[q] = hv[32 * q];
+        d0 = fmaf(b[q], y[0][q], d0);
+        d1 = fmaf(b[q], y[1][q], d1);
+      }
+      const float s = js[Q_HC + k];
+      d0 = -s * warp_sum(d0);
+      if (two) d1 = -s * warp_sum(d1);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        y[0][q] = fmaf(d0, b[q], y[0][q]);
+        if (two) y[1][q] = fmaf(d1, b[q], y[1][q]);
+      }
+    }
+#pragma unroll
+    for (int sl = 0; sl < 2; ++sl) {
+      const int j = warp + 16 * sl;
+      if (j >= r) break;
+      float best = fabsf(y[sl][0]), val = y[sl][0];
+      int bi = lane;
+#pragma unroll
+      for (int q = 1; q < 4; ++q)
+        if (fabsf(y[sl][q]) > best) {
+          best = fabsf(y[sl][q]);
+          val = y[sl][q];
+          bi = lane + 32 * q;
+        }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, o), ov = __shfl_xor_sync(0xFFFFFFFFu, val, o);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) {
+          best = ob;
+          val = ov;
+          bi = oi;
+        }
+      }
+      const float sg = val < 0.0f ? -1.0f : 1.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        U[((size_t)h * 128 + lane + 32 * q) * r + j] = __float2bfloat16_rn(sg * y[sl][q]);
+    }
   }
 }
 
@@ -505,28 +815,10 @@ QWM_API qwm_status qwm_query_basis(const qwm_config* cfg, const void* stats, flo
   __nv_bfloat16* Ub = (U && r > 0) ? static_cast<__nv_bfloat16*>(U) : nullptr;
   const int eig = (Ub || eigenvalues) ? 1 : 0;
   if (!w && !eig) return QWM_OK;
-  // CTAs per head share the rows of V: 4, 2 or 1, one CTA per SM
-  const int sms = sm_count();
-  int SJ = 4;
-  while (SJ > 1 && (int64_t)H * SJ > sms) SJ /= 2;
-  if (!eig) SJ = 1;
-  const int smem = basis_smem_bytes(128 / SJ);
-  if (cudaFuncSetAttribute(basis_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(basis_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBasisSmem) != cudaSuccess)
     return QWM_ERR_CUDA;
-  cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3((unsigned)SJ, (unsigned)H);
-  lc.blockDim = dim3(kJThreads);
-  lc.dynamicSmemBytes = (size_t)smem;
-  lc.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)SJ;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  lc.attrs = at;
-  lc.numAttrs = 1;
   uint8_t* st = static_cast<uint8_t*>(const_cast<void*>(stats));
-  if (cudaLaunchKernelEx(&lc, basis_kernel, st, w, Ub, eigenvalues, r, eig) != cudaSuccess) return QWM_ERR_CUDA;
+  basis_kernel<<<H, kBThreads, kBasisSmem, static_cast<cudaStream_t>(stream)>>>(st, w, Ub, eigenvalues, r, eig);
   return cudaGetLastError() == cudaSuccess ? QWM_OK : QWM_ERR_CUDA;
 }
 
