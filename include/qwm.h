@@ -294,7 +294,7 @@ QWM_API qwm_status qwm_attend_ws(const qwm_config* cfg, const qwm_cache* cache, 
  * qwm_query_stats_bytes(cfg) bytes, 256-byte aligned:
  *   byte 0    int32 device status word (QWM_OK or the first kernel error)
  *   byte 8    uint64 Query count N_<t (tokens folded in so far)
- *   byte 16   int32 Jacobi sweeps of the last qwm_query_basis (maximum over heads)
+ *   byte 16   int32 iterations of qwm_query_basis's eigen-solver (maximum over heads)
  *   byte 256  fp32 sums S_h = sum over past Queries of q q^T, [H][d][d] row-major.
  * --------------------------------------------------------------------------- */
 
@@ -316,13 +316,14 @@ QWM_API qwm_status qwm_query_stats_update(const qwm_config* cfg, void* stats, co
  *      when count = 0 or the mean is 0 (App. C.3 cold start).
  *   U: bf16 [H][d][r], r = cfg->psac_rank (not written when r = 0): the
  *      eigenvectors of M_h for its r largest eigenvalues (Eq. 15), column j
- *      for the j-th largest (equal eigenvalues in increasing index order), each
+ *      for the j-th largest (a diagonal matrix: equal eigenvalues in increasing index order), each
  *      signed so that its largest-magnitude entry (the first such) is positive;
  *      0 when count = 0.
  *   eigenvalues: fp32 [H][d], all eigenvalues of M_h in decreasing order.
- * Any of w, U, eigenvalues may be NULL.  The eigen-solver is cyclic Jacobi in
- * fp32 on the whole 128 x 128 matrix, run until a sweep finds no off-diagonal
- * entry above 2^-20 of the Frobenius norm (at most 30 sweeps). */
+ * Any of w, U, eigenvalues may be NULL.  The eigen-solver works in fp32 on the
+ * whole 128 x 128 matrix: Householder tridiagonalisation, multisection and
+ * inverse iteration; a matrix with no off-diagonal entry above 2^-20 of the
+ * Frobenius norm counts as diagonal. */
 QWM_API qwm_status qwm_query_basis(const qwm_config* cfg, const void* stats, float* w, void* U, float* eigenvalues,
                                    void* stream);
 

@@ -467,7 +467,7 @@ class QueryStats:
         return st.value, cnt.value
 
     def sweeps(self) -> int:
-        """Jacobi sweeps of the last basis computation (maximum over heads)."""
+        """Iterations of the basis computation's eigen-solver (maximum over heads)."""
         return int(self.buffer[16:20].view(torch.int32).item())
 
 

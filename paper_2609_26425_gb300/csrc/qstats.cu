@@ -15,6 +15,8 @@
 //                 leading eigenvectors of M = S / count in fp32 (Eq. 15):
 //                 Householder tridiagonalisation, multisection, inverse
 //                 iteration, back-transformation; one CTA per head.
+#include <type_traits>
+
 #include "qwm_internal.cuh"
 #include "ptx_sm103.cuh"
 
@@ -195,6 +197,11 @@ constexpr int kBasisSmem = (Q_ORD + 128) * 4;
 constexpr int kIter = 2;                         // steps of inverse iteration
 constexpr float kTinyPivot = 1.1920929e-7f;      // 2^-23 of the matrix norm
 
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
@@ -203,44 +210,53 @@ __device__ __forceinline__ float warp_sum(float x) {
 
 // Number of eigenvalues of the tridiagonal T (norm <= 1) below x: sign changes
 // of the leading principal minors p_i = (d_i - x) p_(i-1) - e_(i-1)^2 p_(i-2).
-// A ratio p_i / p_(i-1) below 2^-26 in magnitude is taken as +2^-26 (d_i moved
-// by less than fp32's rounding of the matrix), which keeps four steps between
-// two rescalings inside the fp32 range.
+// e^2 is at least 2^-60 (e moved by less than fp32's rounding of the matrix),
+// so a minor that is exactly zero is followed by one that is not, and four
+// steps between two rescalings stay inside the fp32 range.
 __device__ __forceinline__ int sturm_count(const float* d, const float* e2, float x) {
   float p0 = 0.0f, p1 = 1.0f;
   int n = 0;
 #pragma unroll 1
-  for (int i = 0; i < 128; i += 4) {
-    const float4 dv = *reinterpret_cast<const float4*>(d + i);
-    const float4 ev = *reinterpret_cast<const float4*>(e2 + i);   // e2[i] couples i - 1 and i; e2[0] = 0
-    const float dd[4] = {dv.x, dv.y, dv.z, dv.w}, ee[4] = {ev.x, ev.y, ev.z, ev.w};
+  for (int j = 0; j < 128; j += 32) {
+    uint32_t chg = 0u;   // one bit per step
+#pragma unroll 4
+    for (int i = j; i < j + 32; i += 4) {
+      const float4 dv = *reinterpret_cast<const float4*>(d + i);
+      const float4 ev = *reinterpret_cast<const float4*>(e2 + i);   // e2[i] couples i - 1 and i
+      const float dd[4] = {dv.x, dv.y, dv.z, dv.w}, ee[4] = {ev.x, ev.y, ev.z, ev.w};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      float p = fmaf(dd[k] - x, p1, -(ee[k] * p0));
-      const float lim = 1.4901161e-8f * p1;
-      p = fabsf(p) < fabsf(lim) ? lim : p;
-      n += (int)((__float_as_uint(p) ^ __float_as_uint(p1)) >> 31);
-      p0 = p1;
-      p1 = p;
+      for (int k = 0; k < 4; ++k) {
+        const float p = fmaf(dd[k] - x, p1, -(ee[k] * p0));
+        chg = __funnelshift_l(__float_as_uint(p) ^ __float_as_uint(p1), chg, 1);
+        p0 = p1;
+        p1 = p;
+      }
+      const uint32_t ex = __float_as_uint(fmaxf(fabsf(p0), fabsf(p1))) >> 23;
+      const float sc = __uint_as_float((254u - ex) << 23);   // 2^-exponent of the larger
+      p0 *= sc;
+      p1 *= sc;
     }
-    const float sc = __uint_as_float((254u - ((__float_as_uint(p1) >> 23) & 0xFFu)) << 23);   // 2^-exponent
-    p0 *= sc;
-    p1 *= sc;
+    n += __popc(chg);
   }
   return n;
 }
 
 // w from the diagonal of S (Eq. 8) and the leading eigenvectors of M = S /
 // count (Eq. 15), one CTA per head: Householder tridiagonalisation with M in
-// registers (thread = row tid / 4, a quarter of its columns), all eigenvalues
-// by multisection on Sturm counts, the r leading vectors by two steps of
-// inverse iteration from fixed pseudo-random vectors (LU with partial pivoting,
-// a thread per vector), each followed by modified Gram-Schmidt in decreasing
-// order (so equal eigenvalues get an orthonormal basis), and the Householder
-// vectors applied back (a warp per vector).  A matrix whose off-diagonal
-// entries are all below 2^-20 of its norm counts as diagonal.
-// Bound by the latency of its serial chain (126 reduction steps of two block
-// barriers, 128-step recurrences): the work is 9 n^3 operations a head.
+// registers (thread = 4 rows x 8 columns), eigenvalues by multisection on
+// Sturm counts, the r leading vectors by two steps of inverse iteration from
+// fixed pseudo-random vectors (LU with partial pivoting, a thread per vector),
+// each followed by modified Gram-Schmidt in decreasing order (so equal
+// eigenvalues get an orthonormal basis), and the Householder vectors applied
+// back.  A matrix whose off-diagonal entries are all below 2^-20 of its norm
+// counts as diagonal.
+// Bound by the latency of its serial chain: at 40 heads 126 reduction steps of
+// 1.7 K cycles (214 K), multisection 42 K, LU 11 K, inverse iteration and
+// Gram-Schmidt 35 K, back-transformation 19 K (r = 16).  With a row and a
+// quarter of its columns per thread a step took 2.1 K cycles: every thread then
+// read 32 values of v and of p from shared memory, 1 K cycles of its bandwidth.
+// Statistics reset, update and basis of the Wan-14B layer: 884 us with cyclic
+// Jacobi (7 sweeps of 127 rounds of 2 K cycles), 189 us.
 __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, float* w, __nv_bfloat16* U, float* evals,
                                                              int r, int eig) {
   extern __shared__ __align__(16) float js[];
@@ -264,24 +280,29 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
   if (!eig) return;
   __syncthreads();
 
-  // ---- M = S / count: row i, columns 4 (c + 4 m) .. + 3
-  const int i = tid >> 2, c = tid & 3;
+  // ---- M = S / count: thread (g, c) holds rows g + 32 s, columns 4 (c + 16 m)
+  // .. + 3 (s < 4, m < 2): as many rows as columns, because every step reads v
+  // and p for the columns from shared memory, 128 bytes a cycle for the whole SM
+  const int g = tid >> 4, c = tid & 15;
   const float inv = cnt ? (float)(1.0 / (double)cnt) : 0.0f;
-  uint64_t a[16];
+  uint64_t a[4][4];
   float top = 0.0f, offmax = 0.0f;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const float4 v = *reinterpret_cast<const float4*>(S + i * 128 + 4 * (c + 4 * m));
-    const float x[4] = {v.x * inv, v.y * inv, v.z * inv, v.w * inv};
+  for (int sl = 0; sl < 4; ++sl)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (4 * (c + 4 * m) + e == i) js[Q_D + i] = x[e];
-      else offmax = fmaxf(offmax, fabsf(x[e]));
-      top = fmaxf(top, fabsf(x[e]));
+    for (int m = 0; m < 2; ++m) {
+      const int i = g + 32 * sl, j0 = 4 * (c + 16 * m);
+      const float4 v = *reinterpret_cast<const float4*>(S + i * 128 + j0);
+      const float x[4] = {v.x * inv, v.y * inv, v.z * inv, v.w * inv};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (j0 + e == i) js[Q_D + i] = x[e];
+        else offmax = fmaxf(offmax, fabsf(x[e]));
+        top = fmaxf(top, fabsf(x[e]));
+      }
+      a[sl][2 * m] = f2pack(x[0], x[1]);
+      a[sl][2 * m + 1] = f2pack(x[2], x[3]);
     }
-    a[2 * m] = f2pack(x[0], x[1]);
-    a[2 * m + 1] = f2pack(x[2], x[3]);
-  }
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
     offmax = fmaxf(offmax, __shfl_xor_sync(0xFFFFFFFFu, offmax, o));
@@ -305,8 +326,8 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
 #pragma unroll
   for (int m = 0; m < 16; ++m) {
     float x0, x1;
-    a[m] = mul2(a[m], f2pack(sc0, sc0));
-    f2unpack(a[m], x0, x1);
+    a[m >> 2][m & 3] = mul2(a[m >> 2][m & 3], f2pack(sc0, sc0));
+    f2unpack(a[m >> 2][m & 3], x0, x1);
     ss = fmaf(x0, x0, fmaf(x1, x1, ss));
   }
   offmax *= sc0;
@@ -344,109 +365,127 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
   // ---- T = Q^T M Q: step k takes row k past the diagonal (x, zero up to k) to
   // beta e_(k+1) with H = I - s v v^T, v = x - beta e_(k+1), s = 1 / (beta (beta
   // - x_(k+1))); p = s A v, K = s p.v / 2, A -= v (p - K v)^T + (p - K v) v^T.
-  float* xb = js + Q_XB;
+  float* xb = js + Q_XB;        // v of the step
   float* pb = xb + 128;
-  auto publish = [&](int k) {   // row k of the current matrix, by its four threads
-    if (i == k) {
+  float* hs = js + Q_RED + 16;  // s of the step
+  // row k (slot E = k / 32, threads g = k % 32) of the current matrix: d_k, e_(k+1) = beta, v and s
+  auto publish = [&](auto slot, int k) {
+    constexpr int E = decltype(slot)::value;
+    if (g != (k & 31)) return;
+    const uint32_t half = 0xFFFFu << (lane & 16);
+    float x[8], sig = 0.0f, alpha = 0.0f;
 #pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        float x[4];
-        f2unpack(a[2 * m], x[0], x[1]);
-        f2unpack(a[2 * m + 1], x[2], x[3]);
-        const int j0 = 4 * (c + 4 * m);
+    for (int m = 0; m < 2; ++m) {
+      f2unpack(a[E][2 * m], x[4 * m], x[4 * m + 1]);
+      f2unpack(a[E][2 * m + 1], x[4 * m + 2], x[4 * m + 3]);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (j0 + e == k) js[Q_D + k] = x[e];
-          if (j0 + e <= k) x[e] = 0.0f;
-        }
-        *reinterpret_cast<float4*>(xb + j0) = make_float4(x[0], x[1], x[2], x[3]);
+      for (int e = 0; e < 4; ++e) {
+        const int j = 4 * (c + 16 * m) + e;
+        if (j == k) js[Q_D + k] = x[4 * m + e];
+        x[4 * m + e] = j > k ? x[4 * m + e] : 0.0f;
+        alpha = j == k + 1 ? x[4 * m + e] : alpha;
+        sig = fmaf(x[4 * m + e], x[4 * m + e], sig);
       }
     }
-  };
-  publish(0);
-  __syncthreads();
-#pragma unroll 1
-  for (int k = 0; k < 126; ++k) {
-    const float4 xq = reinterpret_cast<const float4*>(xb)[lane];
-    const float alpha = xb[k + 1];
-    float sig = fmaf(xq.x, xq.x, fmaf(xq.y, xq.y, fmaf(xq.z, xq.z, xq.w * xq.w)));
-    sig = warp_sum(sig);          // x_(k+1)^2 included
-    const float beta = -copysignf(sqrtf(sig), alpha);
-    const bool refl = sig > 1e-30f;   // entries are at most 1: a smaller row counts as zero
-    const float s = refl ? __fdividef(1.0f, beta * (beta - alpha)) : 0.0f;
-    const float vk1 = alpha - beta;
-    const bool live = warp * 8 + 7 > k;   // this warp still has rows past k
-    uint64_t v[16];
-    float vi = 0.0f, p = 0.0f;
-    if (live) {
-      uint64_t acc0 = 0, acc1 = 0;
 #pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int j0 = 4 * (c + 4 * m);
-        float4 x = *reinterpret_cast<const float4*>(xb + j0);
-        if (j0 == ((k + 1) & ~3)) {
-          const int e = (k + 1) & 3;
-          x.x = e == 0 ? vk1 : x.x;
-          x.y = e == 1 ? vk1 : x.y;
-          x.z = e == 2 ? vk1 : x.z;
-          x.w = e == 3 ? vk1 : x.w;
-        }
-        v[2 * m] = f2pack(x.x, x.y);
-        v[2 * m + 1] = f2pack(x.z, x.w);
-        acc0 = fma2(a[2 * m], v[2 * m], acc0);
-        acc1 = fma2(a[2 * m + 1], v[2 * m + 1], acc1);
+    for (int o = 1; o < 16; o <<= 1) {
+      sig += __shfl_xor_sync(half, sig, o);
+      alpha += __shfl_xor_sync(half, alpha, o);
+    }
+    const bool refl = sig > 1e-30f;   // entries are at most 1: a smaller row counts as zero
+    const float beta = -copysignf(sig * rsqrtf(fmaxf(sig, 1e-30f)), alpha);
+    const float vk1 = alpha - beta;
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const int j0 = 4 * (c + 16 * m);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (j0 + e == k + 1) x[4 * m + e] = vk1;
+      const float4 o = make_float4(x[4 * m], x[4 * m + 1], x[4 * m + 2], x[4 * m + 3]);
+      *reinterpret_cast<float4*>(xb + j0) = o;
+      if (k < 126) *reinterpret_cast<float4*>(js + Q_HV + k * 128 + j0) = o;   // for the back-transformation
+    }
+    if (c == 0) {
+      const float s = refl ? __fdividef(1.0f, beta * (beta - alpha)) : 0.0f;
+      hs[0] = s;
+      js[Q_HC + k] = s;
+      if (k < 127) js[Q_E + k + 1] = k == 126 ? alpha : (refl ? beta : 0.0f);
+    }
+  };
+  // steps 32 E .. 32 E + 31: rows of the slots before E and, from E = 2, columns below 64 are done
+  auto segment = [&](auto slot) {
+    constexpr int E = decltype(slot)::value, M0 = E >> 1;
+#pragma unroll 1
+    for (int k = 32 * E; k < (E == 3 ? 126 : 32 * E + 32); ++k) {
+      const float s = hs[0];
+      uint64_t v[4];
+#pragma unroll
+      for (int m = M0; m < 2; ++m) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(xb + 4 * (c + 16 * m));
+        v[2 * m] = t.x;
+        v[2 * m + 1] = t.y;
       }
-      vi = i == k + 1 ? vk1 : xb[i];
-      float y0, y1, y2, y3;
-      f2unpack(acc0, y0, y1);
-      f2unpack(acc1, y2, y3);
-      p = (y0 + y1) + (y2 + y3);
-      p += __shfl_xor_sync(0xFFFFFFFFu, p, 1);
-      p += __shfl_xor_sync(0xFFFFFFFFu, p, 2);
-      p = i > k ? p * s : 0.0f;
-      float kp = p * vi;   // the same in the four threads of a row
+      float p[4] = {0.0f, 0.0f, 0.0f, 0.0f}, vr[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+      for (int sl = E; sl < 4; ++sl) {
+        vr[sl] = xb[g + 32 * sl];
+        uint64_t acc = 0;
+#pragma unroll
+        for (int q = 2 * M0; q < 4; ++q) acc = fma2(a[sl][q], v[q], acc);
+        float y0, y1;
+        f2unpack(acc, y0, y1);
+        p[sl] = y0 + y1;
+      }
+      // sums over the 16 threads of a row, a row slot per lane quarter: lane bits 3, 2 = slot
+      const bool b3 = lane & 8, b2 = lane & 4;
+      float u0 = b3 ? p[2] : p[0], u1 = b3 ? p[3] : p[1];
+      u0 += __shfl_xor_sync(0xFFFFFFFFu, b3 ? p[0] : p[2], 8);
+      u1 += __shfl_xor_sync(0xFFFFFFFFu, b3 ? p[1] : p[3], 8);
+      float pr = b2 ? u1 : u0;
+      pr += __shfl_xor_sync(0xFFFFFFFFu, b2 ? u0 : u1, 4);
+      pr += __shfl_xor_sync(0xFFFFFFFFu, pr, 2);
+      pr += __shfl_xor_sync(0xFFFFFFFFu, pr, 1);
+      const int sl_of = (lane >> 2) & 3, i = g + 32 * sl_of;
+      pr = i > k ? pr * s : 0.0f;
+      if ((lane & 3) == 0) pb[i] = pr;
+      float kp = pr * (b3 ? (b2 ? vr[3] : vr[2]) : (b2 ? vr[1] : vr[0]));
       kp += __shfl_xor_sync(0xFFFFFFFFu, kp, 4);
       kp += __shfl_xor_sync(0xFFFFFFFFu, kp, 8);
       kp += __shfl_xor_sync(0xFFFFFFFFu, kp, 16);
       if (lane == 0) red[warp] = kp;
-      if (c == 0) pb[i] = p;
-    } else {
-      if (lane == 0) red[warp] = 0.0f;
-      if (c == 0) pb[i] = 0.0f;
-    }
-    if (tid < 128) js[Q_HV + k * 128 + tid] = tid == k + 1 ? vk1 : xb[tid];
-    if (tid == 0) {
-      js[Q_HC + k] = s;
-      js[Q_E + k + 1] = refl ? beta : 0.0f;
-    }
-    __syncthreads();
-    if (live) {
-      float K = 0.0f;
+      __syncthreads();
+      float K = red[lane & 15];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 t = reinterpret_cast<const float4*>(red)[q];
-        K += (t.x + t.y) + (t.z + t.w);
-      }
-      K *= 0.5f * s;
-      const float wi = fmaf(-K, vi, p);
-      const uint64_t nK = f2pack(-K, -K), nv = f2pack(-vi, -vi), nw = f2pack(-wi, -wi);
+      for (int o = 1; o < 16; o <<= 1) K += __shfl_xor_sync(0xFFFFFFFFu, K, o);
+      K *= -0.5f * s;
+      const uint64_t nK = f2pack(K, K);
+      uint64_t w2[4];
 #pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const float4 q = *reinterpret_cast<const float4*>(pb + 4 * (c + 4 * m));
-        const uint64_t w0 = fma2(nK, v[2 * m], f2pack(q.x, q.y)), w1 = fma2(nK, v[2 * m + 1], f2pack(q.z, q.w));
-        a[2 * m] = fma2(nv, w0, fma2(nw, v[2 * m], a[2 * m]));
-        a[2 * m + 1] = fma2(nv, w1, fma2(nw, v[2 * m + 1], a[2 * m + 1]));
+      for (int m = M0; m < 2; ++m) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(pb + 4 * (c + 16 * m));
+        w2[2 * m] = fma2(nK, v[2 * m], t.x);
+        w2[2 * m + 1] = fma2(nK, v[2 * m + 1], t.y);
       }
+#pragma unroll
+      for (int sl = E; sl < 4; ++sl) {
+        const float wi = fmaf(K, vr[sl], pb[g + 32 * sl]);
+        const uint64_t nv = f2pack(-vr[sl], -vr[sl]), nw = f2pack(-wi, -wi);
+#pragma unroll
+        for (int q = 2 * M0; q < 4; ++q) a[sl][q] = fma2(nv, w2[q], fma2(nw, v[q], a[sl][q]));
+      }
+      if (E < 3 && k == 32 * E + 31) publish(std::integral_constant<int, (E < 3 ? E + 1 : 3)>(), k + 1);
+      else publish(slot, k + 1);
+      __syncthreads();
     }
-    publish(k + 1);
-    __syncthreads();
-  }
-  if (tid == 0) {
-    js[Q_E + 127] = xb[127];   // row 126 past the diagonal
-    js[Q_E] = 0.0f;
-  }
+  };
+  publish(std::integral_constant<int, 0>(), 0);
   __syncthreads();
-  publish(127);
+  segment(std::integral_constant<int, 0>());
+  segment(std::integral_constant<int, 1>());
+  segment(std::integral_constant<int, 2>());
+  segment(std::integral_constant<int, 3>());
+  publish(std::integral_constant<int, 3>(), 127);
+  if (tid == 0) js[Q_E] = 0.0f;
   __syncthreads();
 
   // ---- scale T to norm <= 1 (a power of two), Gershgorin bounds
@@ -471,40 +510,51 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
     const float e = js[Q_E + tid] * scale;
     js[Q_D + tid] *= scale;
     js[Q_E + tid] = e;
-    js[Q_E2 + tid] = e * e;
+    js[Q_E2 + tid] = fmaxf(e * e, 8.6736174e-19f);   // 2^-60 (see sturm_count)
   }
   lo = lo * scale - 1e-6f;
   hi = hi * scale + 1e-6f;
   __syncthreads();
 
-  // ---- eigenvalues: counts at 512 points, then five-fold sections of each
-  // one's interval by a quad of threads
+  // ---- eigenvalues: counts at a grid of points, then each one's interval in
+  // sections, a point per thread: all 128 (four threads each) when they are
+  // asked for, else the r largest by 128 threads (a warp per sub-partition:
+  // the counts of 16 warps are bound by issue, those of four by latency)
   {
     const float* d = js + Q_D;
     const float* e2 = js + Q_E2;
     int* gc = reinterpret_cast<int*>(js + Q_CNT);
-    const float st = (hi - lo) * (1.0f / 513.0f);
-    gc[tid] = sturm_count(d, e2, fmaf(st, (float)(tid + 1), lo));
+    const int np = evals ? 512 : 128;                       // threads at work, and grid points
+    const int per = evals ? 4 : r > 16 ? 4 : r > 8 ? 8 : 16;  // threads per eigenvalue
+    const float st = (hi - lo) / (float)(np + 1);
+    if (tid < np) gc[tid] = sturm_count(d, e2, fmaf(st, (float)(tid + 1), lo));
     __syncthreads();
-    const int idx = 127 - i;   // eigenvalue i of the decreasing order is number idx of the increasing one
-    int g0 = 0, g1 = 512;      // first grid point with more than idx eigenvalues below it
-    while (g0 < g1) {
-      const int mid = (g0 + g1) >> 1;
-      if (gc[mid] > idx) g1 = mid;
-      else g0 = mid + 1;
-    }
-    float l = g0 == 0 ? lo : fmaf(st, (float)g0, lo), u = g0 == 512 ? hi : fmaf(st, (float)(g0 + 1), lo);
+    if (tid < np) {
+      const int ev = tid / per, q = tid & (per - 1);
+      const int idx = 127 - ev;   // eigenvalue ev of the decreasing order is number idx of the increasing one
+      int g0 = 0, g1 = np;        // first grid point with more than idx eigenvalues below it
+      while (g0 < g1) {
+        const int mid = (g0 + g1) >> 1;
+        if (gc[mid] > idx) g1 = mid;
+        else g0 = mid + 1;
+      }
+      float l = g0 == 0 ? lo : fmaf(st, (float)g0, lo), u = g0 == np ? hi : fmaf(st, (float)(g0 + 1), lo);
+      const float part = 1.0f / (float)(per + 1);
+      // until the interval is below 2^-24: 2 / 513 / 5^7, 2 / 129 / 5^8, 9^6, 17^5
+      const int rounds = evals ? 7 : per == 4 ? 8 : per == 8 ? 6 : 5;
 #pragma unroll 1
-    for (int it = 0; it < 7; ++it) {   // 2 / 513 / 5^7 < 2^-24
-      const float wd = (u - l) * 0.2f;
-      const float x = fmaf(wd, (float)(c + 1), l);
-      const uint32_t above = __ballot_sync(0xFFFFFFFFu, sturm_count(d, e2, x) > idx) >> (lane & 28);
-      const int first = __ffs((int)((above & 15u) | 16u)) - 1;   // section of the quad that holds the eigenvalue
-      const float nl = first == 0 ? l : fmaf(wd, (float)first, l);
-      u = first == 4 ? u : fmaf(wd, (float)(first + 1), l);
-      l = nl;
+      for (int it = 0; it < rounds; ++it) {
+        const float wd = (u - l) * part;
+        const float x = fmaf(wd, (float)(q + 1), l);
+        const uint32_t above = __ballot_sync(0xFFFFFFFFu, sturm_count(d, e2, x) > idx) >> (lane & ~(per - 1));
+        const uint32_t all = (1u << per) - 1u;
+        const int first = __ffs((int)((above & all) | (all + 1u))) - 1;   // section that holds the eigenvalue
+        const float nl = first == 0 ? l : fmaf(wd, (float)first, l);
+        u = first == per ? u : fmaf(wd, (float)(first + 1), l);
+        l = nl;
+      }
+      if (q == 0) js[Q_LAM + ev] = 0.5f * (l + u);
     }
-    if (c == 0) js[Q_LAM + i] = 0.5f * (l + u);
   }
   __syncthreads();
   if (warp == 0) {   // rounding may not put a value above the one before it
@@ -540,29 +590,20 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
     float D = js[Q_D] - lam, Us = js[Q_E + 1];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-#pragma unroll 1
+#pragma unroll 4
       for (int b = 0; b < 32; ++b) {
         const int n = 32 * q + b;
         if (n == 127) break;
         const float e = js[Q_E + n + 1], dn = js[Q_D + n + 1] - lam, en = n < 126 ? js[Q_E + n + 2] : 0.0f;
-        float piv, m1, m2, l;
-        if (fabsf(D) >= fabsf(e)) {
-          piv = fabsf(D) < kTinyPivot ? copysignf(kTinyPivot, D) : D;
-          l = __fdividef(e, piv);
-          m1 = Us;
-          m2 = 0.0f;
-          D = fmaf(-l, Us, dn);
-          Us = en;
-        } else {
-          piv = fabsf(e) < kTinyPivot ? copysignf(kTinyPivot, e) : e;
-          l = __fdividef(D, piv);
-          m1 = dn;
-          m2 = en;
-          D = fmaf(-l, dn, Us);
-          Us = -l * en;
-          swp[q] |= 1u << b;
-        }
-        fi[n * kVecs + lane] = __fdividef(1.0f, piv);
+        const bool s1 = fabsf(D) < fabsf(e);
+        float piv = s1 ? e : D;
+        piv = fabsf(piv) < kTinyPivot ? copysignf(kTinyPivot, piv) : piv;
+        const float rp = rcp_approx(piv), l = (s1 ? D : e) * rp;
+        const float m1 = s1 ? dn : Us, m2 = s1 ? en : 0.0f;
+        D = fmaf(-l, m1, s1 ? Us : dn);
+        Us = s1 ? -l * en : en;
+        swp[q] |= (s1 ? 1u : 0u) << b;
+        fi[n * kVecs + lane] = rp;
         f1[n * kVecs + lane] = m1;
         f2[n * kVecs + lane] = m2;
         fl[n * kVecs + lane] = l;
@@ -584,154 +625,191 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
     X[(e / kVecs) * kXs + (e % kVecs)] = __uint_as_float((z & 0x807FFFFFu) | (107u << 23));
   }
   __syncthreads();
-  float y[2][4];   // warp wq's vectors wq and wq + 16: entries lane + 32 q
+  // From here each vector lives in eight lanes (vector tid / 8, entries 4 (p +
+  // 8 m) .. + 3, p = tid % 8): three shuffle steps a sum and few warps on the
+  // shuffle and shared-memory pipes.
+  const int vec = tid >> 3, vp = tid & 7, nact = r * 8;   // nact threads hold vectors (whole warps)
+  auto sum8 = [](float x) {
+    x += __shfl_xor_sync(0xFFFFFFFFu, x, 1);
+    x += __shfl_xor_sync(0xFFFFFFFFu, x, 2);
+    x += __shfl_xor_sync(0xFFFFFFFFu, x, 4);
+    return x;
+  };
+  float y[16];
 #pragma unroll 1
   for (int it = 0; it < kIter; ++it) {
     if (warp == 0 && lane < r) {
+      // eight steps' operands are loaded before the chain runs through them
       float bc = X[lane];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const uint32_t sw = swp[q];
-#pragma unroll 4
-        for (int b = 0; b < 32; ++b) {
-          const int n = 32 * q + b;
-          if (n < 127) {
-            const float nx = X[(n + 1) * kXs + lane], l = fl[n * kVecs + lane];
-            const bool s1 = (sw >> b) & 1u;
-            const float keep = s1 ? nx : bc, other = s1 ? bc : nx;
-            X[n * kXs + lane] = keep;
-            bc = fmaf(-l, keep, other);
+        uint32_t sw = swp[q];
+#pragma unroll 1
+        for (int b0 = 32 * q; b0 < 32 * q + 32; b0 += 8) {
+          float nx[8], l[8];
+#pragma unroll
+          for (int b = 0; b < 8; ++b) {
+            const int n = min(b0 + b, 126);
+            nx[b] = X[(n + 1) * kXs + lane];
+            l[b] = fl[n * kVecs + lane];
           }
+#pragma unroll
+          for (int b = 0; b < 8; ++b) {
+            if (b0 + b < 127) {
+              const bool s1 = (sw >> b) & 1u;
+              const float keep = s1 ? nx[b] : bc, other = s1 ? bc : nx[b];
+              X[(b0 + b) * kXs + lane] = keep;
+              bc = fmaf(-l[b], keep, other);
+            }
+          }
+          sw >>= 8;
         }
       }
+      X[127 * kXs + lane] = bc;
       float x1 = 0.0f, x2 = 0.0f;
-#pragma unroll 4
-      for (int n = 127; n >= 0; --n) {
-        const float b = n == 127 ? bc : X[n * kXs + lane];
-        const float x0 = fmaf(-f1[n * kVecs + lane], x1, fmaf(-f2[n * kVecs + lane], x2, b)) * fi[n * kVecs + lane];
-        X[n * kXs + lane] = x0;
-        x2 = x1;
-        x1 = x0;
+#pragma unroll 1
+      for (int n0 = 120; n0 >= 0; n0 -= 8) {
+        float b[8], u1[8], u2[8], ip[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int n = n0 + k;
+          b[k] = X[n * kXs + lane];
+          u1[k] = f1[n * kVecs + lane];
+          u2[k] = f2[n * kVecs + lane];
+          ip[k] = fi[n * kVecs + lane];
+        }
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+          const float x0 = fmaf(-u1[k], x1, fmaf(-u2[k], x2, b[k])) * ip[k];
+          X[(n0 + k) * kXs + lane] = x0;
+          x2 = x1;
+          x1 = x0;
+        }
       }
     }
     __syncthreads();
     // modified Gram-Schmidt, largest eigenvalue first
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-      const int j = warp + 16 * sl;
+    if (tid < nact) {
       float mx = 0.0f;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        y[sl][q] = j < r ? X[(lane + 32 * q) * kXs + j] : 0.0f;
-        mx = fmaxf(mx, fabsf(y[sl][q]));
+      for (int m = 0; m < 16; ++m) {
+        y[m] = X[(4 * (vp + 8 * (m >> 2)) + (m & 3)) * kXs + vec];
+        mx = fmaxf(mx, fabsf(y[m]));
       }
 #pragma unroll
-      for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+      for (int o = 4; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
       const float sc = mx > 0.0f && mx < INFINITY ? __fdividef(1.0f, mx) : 0.0f;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) y[sl][q] = fabsf(y[sl][q]) < INFINITY ? y[sl][q] * sc : 0.0f;
-    }
+      for (int m = 0; m < 16; ++m) y[m] = fabsf(y[m]) < INFINITY ? y[m] * sc : 0.0f;
+      // a second pass when a vector lost most of its length in the first (its
+      // direction is then no longer orthogonal to fp32)
+      float n0 = 0.0f;
+#pragma unroll
+      for (int m = 0; m < 16; ++m) n0 = fmaf(y[m], y[m], n0);
+      n0 = sum8(n0);
+      bool lost = false;
 #pragma unroll 1
-    for (int j = 0; j < r; ++j) {
-      float* vb = xb + 128 * (j & 1);
-      const int own = j >> 4;
-      if (warp == (j & 15)) {
+      for (int j = 0; j < r; ++j) {
+        float4* vb = reinterpret_cast<float4*>(xb + 128 * (j & 1)) + vp;
+        if (warp == (j >> 2)) {   // the vector's eight lanes are in this warp
+          float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int sl = 0; sl < 2; ++sl)
-          if (sl == own) {
-            float n2 = 0.0f;
+          for (int m = 0; m < 16; ++m) s4[m & 3] = fmaf(y[m], y[m], s4[m & 3]);
+          const float n2 = sum8((s4[0] + s4[1]) + (s4[2] + s4[3]));
+          if (vec == j) {
+            const float sc1 = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
+            lost |= n2 < 1e-2f * n0;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) n2 = fmaf(y[sl][q], y[sl][q], n2);
-            n2 = warp_sum(n2);
-            const float sc = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
+            for (int m = 0; m < 16; ++m) y[m] *= sc1;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              y[sl][q] *= sc;
-              vb[lane + 32 * q] = y[sl][q];
-            }
+            for (int m = 0; m < 4; ++m) vb[8 * m] = make_float4(y[4 * m], y[4 * m + 1], y[4 * m + 2], y[4 * m + 3]);
           }
-      }
-      __syncthreads();
+        }
+        named_bar_sync(1, nact);
+        if (warp >= (j >> 2)) {
+          float b[16], s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int sl = 0; sl < 2; ++sl) {
-        const int k = warp + 16 * sl;
-        if (k > j && k < r) {
-          float dt = 0.0f, b[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            b[q] = vb[lane + 32 * q];
-            dt = fmaf(b[q], y[sl][q], dt);
+          for (int m = 0; m < 4; ++m) {
+            const float4 t = vb[8 * m];
+            b[4 * m] = t.x; b[4 * m + 1] = t.y; b[4 * m + 2] = t.z; b[4 * m + 3] = t.w;
           }
-          dt = warp_sum(dt);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) y[sl][q] = fmaf(-dt, b[q], y[sl][q]);
+          for (int m = 0; m < 16; ++m) s4[m & 3] = fmaf(b[m], y[m], s4[m & 3]);
+          const float dt = sum8((s4[0] + s4[1]) + (s4[2] + s4[3]));
+          if (vec > j)
+#pragma unroll
+            for (int m = 0; m < 16; ++m) y[m] = fmaf(-dt, b[m], y[m]);
+        }
+        if (j == r - 1 && named_bar_or(1, nact, lost)) {
+          j = -1;
+          n0 = 0.0f;
+          lost = false;
         }
       }
-    }
-    if (it + 1 < kIter) {
+      if (it + 1 < kIter)
 #pragma unroll
-      for (int sl = 0; sl < 2; ++sl) {
-        const int j = warp + 16 * sl;
-        if (j < r)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) X[(lane + 32 * q) * kXs + j] = y[sl][q] * 9.5367432e-7f;
-      }
+        for (int m = 0; m < 16; ++m) X[(4 * (vp + 8 * (m >> 2)) + (m & 3)) * kXs + vec] = y[m] * 9.5367432e-7f;
     }
     __syncthreads();
   }
+  if (tid >= nact) return;
 
-  // ---- back to M's coordinates: H_0 ... H_125 y; then the sign rule (the
-  // largest |entry|, the first one on ties, is positive) and bf16
-  const bool two = warp + 16 < r;
-  if (warp < r) {
-    const float* hv = js + Q_HV + 125 * 128 + lane;
-#pragma unroll 2
-    for (int k = 125; k >= 0; --k, hv -= 128) {
-      float b[4], d0 = 0.0f, d1 = 0.0f;
+  // ---- back to M's coordinates: H_0 ... H_125 y, two reflections at a time:
+  // H_(k-1) H_k y needs v_k.y, v_(k-1).y and v_(k-1).v_k, whose sums run together
+  const float4* hv = reinterpret_cast<const float4*>(js + Q_HV + 125 * 128) + vp;
+#pragma unroll 1
+  for (int k = 125; k > 0; k -= 2, hv -= 64) {
+    float b[16], g[16], d4[4] = {0.0f, 0.0f, 0.0f, 0.0f}, g4[4] = {0.0f, 0.0f, 0.0f, 0.0f}, q4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        b[q] = hv[32 * q];
-        d0 = fmaf(b[q], y[0][q], d0);
-        d1 = fmaf(b[q], y[1][q], d1);
-      }
-      const float s = js[Q_HC + k];
-      d0 = -s * warp_sum(d0);
-      if (two) d1 = -s * warp_sum(d1);
+    for (int m = 0; m < 4; ++m) {
+      const float4 t = hv[8 * m], u = hv[8 * m - 32];
+      b[4 * m] = t.x; b[4 * m + 1] = t.y; b[4 * m + 2] = t.z; b[4 * m + 3] = t.w;
+      g[4 * m] = u.x; g[4 * m + 1] = u.y; g[4 * m + 2] = u.z; g[4 * m + 3] = u.w;
+    }
+    const float s = -js[Q_HC + k], t = -js[Q_HC + k - 1];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        y[0][q] = fmaf(d0, b[q], y[0][q]);
-        if (two) y[1][q] = fmaf(d1, b[q], y[1][q]);
-      }
+    for (int m = 0; m < 16; ++m) {
+      d4[m & 3] = fmaf(b[m], y[m], d4[m & 3]);
+      g4[m & 3] = fmaf(g[m], y[m], g4[m & 3]);
+      q4[m & 3] = fmaf(b[m], g[m], q4[m & 3]);
+    }
+    float d0 = (d4[0] + d4[1]) + (d4[2] + d4[3]), g0 = (g4[0] + g4[1]) + (g4[2] + g4[3]);
+    float bg = (q4[0] + q4[1]) + (q4[2] + q4[3]);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      d0 += __shfl_xor_sync(0xFFFFFFFFu, d0, o);
+      g0 += __shfl_xor_sync(0xFFFFFFFFu, g0, o);
+      bg += __shfl_xor_sync(0xFFFFFFFFu, bg, o);
+    }
+    d0 *= s;
+    g0 = t * fmaf(d0, bg, g0);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) y[m] = fmaf(g0, g[m], fmaf(d0, b[m], y[m]));
+  }
+  // the sign rule (the largest |entry|, the first one on ties, is positive) and bf16
+  float best = -1.0f, val = 0.0f;
+  int bi = 0;
+#pragma unroll
+  for (int m = 0; m < 16; ++m)   // ascending entries of this lane
+    if (fabsf(y[m]) > best) {
+      best = fabsf(y[m]);
+      val = y[m];
+      bi = 4 * (vp + 8 * (m >> 2)) + (m & 3);
     }
 #pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-      const int j = warp + 16 * sl;
-      if (j >= r) break;
-      float best = fabsf(y[sl][0]), val = y[sl][0];
-      int bi = lane;
-#pragma unroll
-      for (int q = 1; q < 4; ++q)
-        if (fabsf(y[sl][q]) > best) {
-          best = fabsf(y[sl][q]);
-          val = y[sl][q];
-          bi = lane + 32 * q;
-        }
-#pragma unroll
-      for (int o = 16; o; o >>= 1) {
-        const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, o), ov = __shfl_xor_sync(0xFFFFFFFFu, val, o);
-        const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          val = ov;
-          bi = oi;
-        }
-      }
-      const float sg = val < 0.0f ? -1.0f : 1.0f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        U[((size_t)h * 128 + lane + 32 * q) * r + j] = __float2bfloat16_rn(sg * y[sl][q]);
+  for (int o = 1; o < 8; o <<= 1) {
+    const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, o), ov = __shfl_xor_sync(0xFFFFFFFFu, val, o);
+    const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+    if (ob > best || (ob == best && oi < bi)) {
+      best = ob;
+      val = ov;
+      bi = oi;
     }
   }
+  const float sg = val < 0.0f ? -1.0f : 1.0f;
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    U[((size_t)h * 128 + 4 * (vp + 8 * (m >> 2)) + (m & 3)) * r + vec] = __float2bfloat16_rn(sg * y[m]);
 }
 
 int sm_count() {
