@@ -11,19 +11,30 @@
 //   fit_assign  (persistent, one CTA per SM, tcgen05).  A 128-token tile
 //     arrives by TMA and two MMAs per K step accumulate
 //     P = X mu_hi^T + X mu_lo^T in TMEM (mu_hi = bf16(mu), mu_lo =
-//     bf16(mu - mu_hi): mu to 2^-18 relative; bf16 x bf16 products are exact).
-//     With dt_j = |mu_j|^2 - 2 P_j, |dt_j + |x|^2 - d_j| stays below
-//     E = 2^-11 (|x|^2 + max_j |mu_j|^2) for the sequential fp32 distance d_j
-//     (operand split 2^-18, fp32 accumulation of 256 products 2^-15, the
-//     norms and the sequential sum's own rounding (d + 2) 2^-24, each relative
-//     to |x|^2 + |mu_j|^2, with margin).  Every centroid within 2E of the
-//     smallest dt is therefore a candidate for the exact argmin; a row with a
-//     single candidate is decided, the others (a few percent) are rescored
-//     with the sequential fp32 distance.
-//   fit_scatter (one CTA per head): counting sort of the tokens by cluster.
-//   fit_means   (one warp per centroid): exact fp64 member sums (bf16 values
-//     of ordinary range add exactly, so the order does not matter), the mean,
-//     and the next iteration's operand images and norm.
+//     bf16(mu - mu_hi): mu to 2^-18 relative; bf16 x bf16 products are exact);
+//     one more MMA, a column of ones against -|mu_j|^2 / 2 in two bf16 parts,
+//     makes it s_j = P_j - |mu_j|^2 / 2, so that |x|^2 - 2 s_j is the distance
+//     and the row's nearest centroid its largest s_j, which the TMEM load
+//     reduces on its way.  ||x|^2 - 2 s_j - d_j| stays below
+//     E_j = c (|x|^2 + |mu_j|^2), c = 2^-13, for the sequential fp32 distance
+//     d_j: fp32 accumulation of 256 products at two ulps of the running
+//     absolute sum each, 2^-13 |x| |mu_j|; the operand split 2^-18 and the
+//     norm's 2^-17, the fp32 norms and the sequential sum's own rounding
+//     2^-16, all relative to |x|^2 + |mu_j|^2: 0.75 c.  With k the largest
+//     computed s and j the exact argmin, E_j + E_k bounds 2 (s_k - s_j), and
+//     both centroids are within (|x| + sqrt(d))^2 <= 2 (|x|^2 + d) of the origin
+//     squared, d = |x|^2 - 2 s_k the distance found (+ E): so every j with
+//     s_j > s_k - c (|x|^2 + 2.02 (|x|^2 + d)) is a candidate for the exact
+//     argmin.  A row with a single candidate is decided, the others are
+//     rescored with the sequential fp32 distance.
+//   fit_means   (four warps per centroid): the members of a centroid are picked
+//     out of the head's assignment bytes (more than kScanTokens tokens: read
+//     from a list that fit_scatter, one CTA per head, sorts by cluster); exact
+//     member sums (bf16 values of ordinary range add exactly, so the order does
+//     not matter), the mean, and the next iteration's operand images and norm;
+//     the last iteration's launch writes the bf16 result.
+// Each launch is a programmatic dependent of the one before it (its prologue
+// overlaps that one's tail).
 #include <mutex>
 
 #include "ptx_sm103.cuh"
@@ -34,6 +45,7 @@ namespace {
 
 using namespace ptx;
 
+constexpr int kScanTokens = 8192;             // tokens up to which fit_means scans the assignment (fit_carve)
 constexpr int AT = 128;                       // tokens per tile
 constexpr int AEW = 16;                       // epilogue warps: rows 32 (w & 3) + lane, column quarter w >> 2
 constexpr int ANT = (AEW + 1) * 32;           // + one producer / MMA warp
@@ -41,15 +53,38 @@ constexpr int kPairCap = 1024;                // (row, centroid) pairs rescored 
 constexpr int kRowCap = 8;                    // candidates per row
 constexpr int A_X = 0;                        // 2 token tiles, each 2 x [128 rows][128 B] bf16
 constexpr int A_IMG = 65536;                  // operand images hi, lo: 2 x 2 x [Npad][128 B]
-constexpr int A_NRM = A_IMG + 131072;         // |mu_j|^2 [256] for each TMEM buffer
-constexpr int A_PJ = A_NRM + 2048;            // pair (row << 16 | j) [kPairCap]
+constexpr int A_ONE = A_IMG + 131072;         // ones: [128 rows][16] bf16 operand (columns 0 and 1), no swizzle
+constexpr int A_NRM = A_ONE + 4096;           // -|mu_j|^2 / 2 in two bf16 parts: [256 rows][16], no swizzle
+constexpr int A_PJ = A_NRM + 8192;            // pair (row << 16 | j) [kPairCap]
 constexpr int A_PD = A_PJ + kPairCap * 4;     // pair distance [kPairCap]
 constexpr int A_ROW = A_PD + kPairCap * 4;    // row: first slot << 16 | count (0xFFFF: full scan)
-constexpr int A_MIN = A_ROW + AT * 4;         // [4 quarters][128] partial minima
-constexpr int A_CNT = A_MIN + 4 * AT * 4;     // [4 quarters][128] candidate counts
+constexpr int A_MIN = A_ROW + AT * 4;         // [4 quarters][128] partial maxima of s
+constexpr int A_CNT = A_MIN + 4 * AT * 4;     // [4 quarters][128] candidate count | first candidate << 8
 constexpr int A_CND = A_CNT + 4 * AT * 4;     // [128][4 quarters][kRowCap] candidates (u8)
 constexpr int A_BAR = A_CND + AT * 4 * kRowCap;   // mbarriers, pair counter, flag, TMEM slot
 constexpr int A_SMEM = A_BAR + 128 + 1024;
+static_assert(A_SMEM <= 232448, "shared memory of the assignment kernel");
+constexpr uint32_t kPadNorm = 0x0000F149u;    // bf16 -1e30 | 0 << 16: a padding column never wins
+
+// Operand block of rows of 16 two-byte values without swizzle: 8 rows x 16
+// bytes contiguous, the second half of the values 128 bytes on, row groups 256
+// bytes apart.
+__device__ __forceinline__ uint64_t desc_k16(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(128u >> 4) << 16;
+  d |= (uint64_t)(256u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+__device__ __forceinline__ int k16_off(int row) { return (row >> 3) * 256 + (row & 7) * 16; }
+
+// -n2 / 2 as two bf16 parts (the first in the low half-word).
+__device__ __forceinline__ uint32_t half_norm(float n2) {
+  const float v = -0.5f * n2;
+  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+  return pack_bf16(v, v - __bfloat162float(hi));
+}
 
 // Byte offset of 16-byte chunk `ch` (channels 8ch..8ch+7) of row `row` in two
 // 128-byte-swizzled blocks of `rows` rows x 64 two-byte elements.
@@ -99,25 +134,31 @@ __device__ __forceinline__ void emit_row(const FitArgs& a, int h, int j, float4 
   float n2 = fmaf(m.x, m.x, fmaf(m.y, m.y, fmaf(m.z, m.z, m.w * m.w)));
 #pragma unroll
   for (int o = 16; o; o >>= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, o);
-  if (lane == 0) {
-    a.nrm[(size_t)h * a.Npad + j] = n2;
-    atomicMax(a.nmax + h, __float_as_uint(n2));  // n2 >= 0: the bits order like the values
-  }
+  if (lane == 0) a.nrm[(size_t)h * a.Npad + j] = half_norm(n2);
 }
 
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Initial centroids (token floor(j N / C)) and their images; padding rows
-// j in [C, Npad) get zero images and norm.  One warp per (head, row).
+// j in [C, Npad) get zero images and norm; the counters start at zero.  One
+// warp per (head, row).
 __global__ void __launch_bounds__(512) fit_prep(const FitArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= (int64_t)a.H * a.Npad) return;
   const int h = (int)(w / a.Npad), j = (int)(w % a.Npad);
+  if (lane == 0) {
+    if (w == 0) *a.status = 0;
+    if (j == 0) a.emax[h] = 0;
+    if (j < a.C) a.counts[(size_t)h * a.C + j] = 0;
+  }
   if (j >= a.C) {
     const size_t off = (size_t)sw_off(a.Npad, j, lane >> 1) + (size_t)(lane & 1) * 8;
     uint8_t* hi = a.img + (size_t)h * 2 * a.Npad * 256;
     *reinterpret_cast<uint2*>(hi + off) = make_uint2(0, 0);
     *reinterpret_cast<uint2*>(hi + (size_t)a.Npad * 256 + off) = make_uint2(0, 0);
-    if (lane == 0) a.nrm[(size_t)h * a.Npad + j] = INFINITY;  // padding columns never win
+    if (lane == 0) a.nrm[(size_t)h * a.Npad + j] = kPadNorm;
     return;
   }
   const int64_t src = ((int64_t)j * a.N) / a.C;
@@ -129,10 +170,11 @@ __global__ void __launch_bounds__(512) fit_prep(const FitArgs a) {
 }
 
 // Assignment of every token (see the file comment).  Units are (head, tile)
-// in head-major order, split into contiguous runs over the CTAs.  Warp 8 loads
+// in head-major order, split into contiguous runs over the CTAs.  Warp 16 loads
 // (TMA) and multiplies (tcgen05) tile t + 1 into the second token buffer and
-// TMEM accumulator while warps 0-7 finish tile t: two warps per row, one per
-// column half of the accumulator, meeting in shared memory.
+// TMEM accumulator while warps 0-15 finish tile t: four warps per row, one per
+// column quarter of the accumulator (at most 64 columns, read once and kept in
+// registers), meeting in shared memory.
 __global__ void __launch_bounds__(ANT, 1)
     fit_assign(const FitArgs a, const __grid_constant__ CUtensorMap tm, int tiles, int units) {
   extern __shared__ uint8_t smem_raw[];
@@ -155,15 +197,22 @@ __global__ void __launch_bounds__(ANT, 1)
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + A_BAR + 72);
   uint32_t ncols = 32;
   while ((int)ncols < Npad) ncols <<= 1;
+  const int Nm = (Npad + 31) & ~31;
 
   if (warp == 0) {
     tmem_alloc(smem_u32(tslot), 2 * ncols);
     tmem_relinquish();
   }
-  // norms past Npad are never copied in: +inf, so that columns beyond the
-  // MMA width (read when Npad is not a multiple of 32) never win
-  for (int i = tid; i < 512; i += ANT)
-    if ((i & 255) >= Npad) reinterpret_cast<float*>(sm + A_NRM)[i] = INFINITY;
+  // the ones operand; the norm operand's unused columns; the image rows from
+  // Npad to the MMA width Nm (a multiple of 32: the loads read whole chunks)
+  for (int i = tid; i < 128 * 2; i += ANT)
+    *reinterpret_cast<uint4*>(sm + A_ONE + i * 16) = make_uint4((i & 8) ? 0u : 0x3F803F80u, 0u, 0u, 0u);
+  for (int i = tid; i < 256 * 2; i += ANT)
+    *reinterpret_cast<uint4*>(sm + A_NRM + i * 16) = make_uint4((i & 8) ? 0u : kPadNorm, 0u, 0u, 0u);
+  for (int i = tid; i < 4 * (Nm - Npad) * 8; i += ANT)
+    *reinterpret_cast<uint4*>(sm + A_IMG + (i / ((Nm - Npad) * 8)) * Nm * 128 + Npad * 128 + (i % ((Nm - Npad) * 8)) * 16) =
+        make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
   if (tid == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar_tma(b), 1);
@@ -178,6 +227,8 @@ __global__ void __launch_bounds__(ANT, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch();
+  pdl_wait();   // the images, norms and member lists of the launches before
   const uint32_t tbase = *tslot;
   const int u0 = (int)((int64_t)blockIdx.x * units / gridDim.x);
   const int u1 = (int)((int64_t)(blockIdx.x + 1) * units / gridDim.x);
@@ -185,31 +236,49 @@ __global__ void __launch_bounds__(ANT, 1)
 
   if (warp == AEW) {
     // ---------------- producer / MMA issuer
-    if (lane == 0) {
-      const uint32_t id = idesc_f16(128, Npad, false, true);
-      const uint32_t aI = smem_u32(sm + A_IMG);
-      const uint32_t ib = (uint32_t)Npad * 512u;
-      int cur_h = -1;
-      uint32_t ph_img = 0;
-      for (int t = 0; t < T; ++t) {
-        const int u = u0 + t, h = u / tiles, tile = u - h * tiles, b = t & 1;
-        if (t >= 2 && !mbar_wait(bar_free(b), ((t >> 1) - 1) & 1)) { *s_err = 1; break; }
-        if (h != cur_h) {
-          // the previous head's MMAs read the images: wait for them, then load this head's
-          if (t >= 1 && !mbar_wait(bar_mma((t - 1) & 1), ((t - 1) >> 1) & 1)) { *s_err = 1; break; }
-          mbar_arrive_expect_tx(bar_img, ib);
-          bulk_g2s(aI, a.img + (size_t)h * ib, ib, bar_img);
-          if (!mbar_wait(bar_img, ph_img)) { *s_err = 1; break; }
+    const uint32_t id = idesc_f16(128, Nm, false, true);
+    const uint32_t aI = smem_u32(sm + A_IMG);
+    int cur_h = -1;
+    uint32_t ph_img = 0;
+    bool go = true;
+    for (int t = 0; t < T && go; ++t) {
+      const int u = u0 + t, h = u / tiles, tile = u - h * tiles, b = t & 1;
+      if (t >= 2) go = __all_sync(0xFFFFFFFFu, mbar_wait(bar_free(b), ((t >> 1) - 1) & 1));
+      const bool copying = go;
+      const uint32_t aX = smem_u32(sm + A_X + b * 32768);
+      if (go && lane == 0) {
+        mbar_arrive_expect_tx(bar_tma(b), 32768u);
+        tma_load_3d(aX, &tm, 0, h, tile * 128, bar_tma(b));
+        tma_load_3d(aX + 16384, &tm, 64, h, tile * 128, bar_tma(b));
+      }
+      if (go && h != cur_h) {
+        // the previous head's MMAs read the images and norms: wait for them, then load this head's
+        if (t >= 1) go = mbar_wait(bar_mma((t - 1) & 1), ((t - 1) >> 1) & 1);
+        go = __all_sync(0xFFFFFFFFu, go);
+        if (go) {
+          if (lane == 0) {
+            mbar_arrive_expect_tx(bar_img, (uint32_t)Npad * 512u);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)   // hi, lo x channels [0, 64), [64, 128)
+              bulk_g2s(aI + q * Nm * 128, a.img + ((size_t)h * 4 + q) * Npad * 128, (uint32_t)Npad * 128u, bar_img);
+          }
+          for (int j = lane; j < Npad; j += 32)
+            *reinterpret_cast<uint32_t*>(sm + A_NRM + k16_off(j)) = a.nrm[(size_t)h * Npad + j];
+          fence_proxy_async_smem();
+          go = mbar_wait(bar_img, ph_img);
           ph_img ^= 1;
           cur_h = h;
         }
-        const uint32_t aX = smem_u32(sm + A_X + b * 32768);
-        mbar_arrive_expect_tx(bar_tma(b), 32768u + (uint32_t)Npad * 4u);
-        tma_load_3d(aX, &tm, 0, h, tile * 128, bar_tma(b));
-        tma_load_3d(aX + 16384, &tm, 64, h, tile * 128, bar_tma(b));
-        bulk_g2s(smem_u32(sm + A_NRM + b * 1024), a.nrm + (size_t)h * Npad, (uint32_t)Npad * 4u, bar_tma(b));
-        if (!mbar_wait(bar_tma(b), (t >> 1) & 1)) { *s_err = 1; break; }
-        tc_fence_after();
+      }
+      if (go) go = mbar_wait(bar_tma(b), (t >> 1) & 1);
+      go = __all_sync(0xFFFFFFFFu, go);
+      if (!go) {
+        if (copying) mbar_wait(bar_tma(b), (t >> 1) & 1);   // no copy outlives the CTA
+        *s_err = 1;
+        break;
+      }
+      tc_fence_after();
+      if (lane == 0) {
         const uint32_t tD = tbase + (uint32_t)b * ncols;
 #pragma unroll
         for (int half = 0; half < 2; ++half)
@@ -217,12 +286,13 @@ __global__ void __launch_bounds__(ANT, 1)
           for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-              umma_ss(tD, desc_sw128(aX + kb * 16384 + ks * 32),
-                      desc_sw128(aI + half * Npad * 256 + kb * Npad * 128 + ks * 32), id, (half | kb | ks) != 0);
+              umma_ss(tD, desc_sw128(aX + kb * 16384 + ks * 32), desc_sw128(aI + (half * 2 + kb) * Nm * 128 + ks * 32),
+                      id, (half | kb | ks) != 0);
+        umma_ss(tD, desc_k16(smem_u32(sm + A_ONE)), desc_k16(smem_u32(sm + A_NRM)), id, 1u);
         umma_commit(bar_mma(b));
       }
+      __syncwarp();
     }
-    __syncwarp();
   } else {
     // ---------------- epilogue: warps 0-15
     const int qt = warp >> 2, row = (warp & 3) * 32 + lane;
@@ -232,7 +302,6 @@ __global__ void __launch_bounds__(ANT, 1)
     for (int t = 0; t < T; ++t) {
       const int u = u0 + t, h = u / tiles, tile = u - h * tiles, b = t & 1;
       const uint8_t* sX = sm + A_X + b * 32768;
-      const float4* sNrm4 = reinterpret_cast<const float4*>(sm + A_NRM + b * 1024);  // +inf past C
       const uint32_t tD = tbase + (uint32_t)b * ncols;
       const int64_t n = (int64_t)tile * 128 + row;
       const bool valid = n < a.N;
@@ -241,81 +310,76 @@ __global__ void __launch_bounds__(ANT, 1)
       ok = __all_sync(0xFFFFFFFFu, ok);
       tc_fence_after();
       if (!ok) *s_err = 1;
-      // smallest dt of this quarter
-      float mn = INFINITY;
-      if (ok) {
-#pragma unroll 1
-        for (int cb = ch0; cb < ch1; cb += 2) {
-          float v[64];
-          const int cb2 = cb + 1 < ch1 ? cb + 1 : cb;  // a lone last chunk is read twice (harmless for a minimum)
-          tmem_ld32x2(tD + lrow + cb * 32, tD + lrow + cb2 * 32, *reinterpret_cast<float(*)[32]>(v),
-                      *reinterpret_cast<float(*)[32]>(v + 32));
-#pragma unroll
-          for (int e4 = 0; e4 < 16; ++e4) {
-            const float4 nr = sNrm4[(e4 < 8 ? cb : cb2) * 8 + (e4 & 7)];
-            mn = fminf(mn, fminf(fminf(fmaf(-2.0f, v[4 * e4], nr.x), fmaf(-2.0f, v[4 * e4 + 1], nr.y)),
-                                 fminf(fmaf(-2.0f, v[4 * e4 + 2], nr.z), fmaf(-2.0f, v[4 * e4 + 3], nr.w))));
-          }
-        }
+      // s_j of this quarter's columns and the largest
+      constexpr float kC = 1.220703125e-4f;   // c
+      float v[64];
+      float mx = -INFINITY;
+      const bool any = ok && ch0 < ch1;
+      if (any) {
+        const int cb2 = ch0 + 1 < ch1 ? ch0 + 1 : ch0;  // a lone chunk is read twice
+        mx = tmem_ld64_max(tD + lrow + ch0 * 32, tD + lrow + cb2 * 32, v);
       }
-      sMin[qt * AT + row] = mn;
-      named_bar_sync(1, AEW * 32);
-      mn = fminf(fminf(sMin[row], sMin[AT + row]), fminf(sMin[2 * AT + row], sMin[3 * AT + row]));
-      const float thr = mn + 2.0f * ldexpf(kx + __uint_as_float(a.nmax[h]), -11);
-      // this quarter's candidates, ascending
-      int cnt = 0;
-      uint8_t* cand = sCnd + (row * 4 + qt) * kRowCap;
-      if (ok && thr < INFINITY) {
-#pragma unroll 1
-        for (int cb = ch0; cb < ch1; cb += 2) {
-          float v[64];
-          const int cb2 = cb + 1 < ch1 ? cb + 1 : cb;
-          tmem_ld32x2(tD + lrow + cb * 32, tD + lrow + cb2 * 32, *reinterpret_cast<float(*)[32]>(v),
-                      *reinterpret_cast<float(*)[32]>(v + 32));
-          const int ne = cb2 > cb ? 64 : 32;
-#pragma unroll
-          for (int e4 = 0; e4 < 16; ++e4) {
-            const float4 nr = sNrm4[(e4 < 8 ? cb : cb2) * 8 + (e4 & 7)];
-            const float d4[4] = {fmaf(-2.0f, v[4 * e4], nr.x), fmaf(-2.0f, v[4 * e4 + 1], nr.y),
-                                 fmaf(-2.0f, v[4 * e4 + 2], nr.z), fmaf(-2.0f, v[4 * e4 + 3], nr.w)};
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (4 * e4 + q < ne && d4[q] <= thr) {
-                if (cnt < kRowCap) cand[cnt] = (uint8_t)(cb * 32 + 4 * e4 + q);
-                ++cnt;
-              }
-          }
-        }
-      }
-      sCnt[qt * AT + row] = (ok && thr < INFINITY) ? cnt : -1;
+      sMin[qt * AT + row] = mx;
       tc_fence_before();
+      named_bar_sync(1, AEW * 32);
+      mx = fmaxf(fmaxf(sMin[row], sMin[AT + row]), fmaxf(sMin[2 * AT + row], sMin[3 * AT + row]));
+      const float dist = fmaxf(fmaf(-2.0f, mx, kx), 0.0f);
+      const float thr = fmaf(-kC, fmaf(2.02f, kx + dist, kx), mx) - 1e-30f;
+      const bool fin = ok && thr > -INFINITY && thr < INFINITY && kx < INFINITY;
+      // this quarter's candidates, ascending (bit 31 - e of a mask: column e)
+      int cnt = 0;
+      uint32_t word = 0xFFu;   // count (0xFF: every centroid), first candidate << 8
+      uint8_t* cand = sCnd + (row * 4 + qt) * kRowCap;
+      if (fin) {
+        uint32_t mk[2] = {0u, 0u};
+        if (any) {
+#pragma unroll
+          for (int e = 0; e < 64; ++e) mk[e >> 5] = __funnelshift_l(__float_as_uint(thr - v[e]), mk[e >> 5], 1);
+          if (ch0 + 1 >= ch1) mk[1] = 0u;
+        }
+        cnt = __popc(mk[0]) + __popc(mk[1]);
+        const int first = mk[0] ? __clz((int)mk[0]) : 32 + __clz((int)mk[1]);
+        word = (uint32_t)cnt | ((uint32_t)(ch0 * 32 + first) << 8);
+        if (cnt > 1) {
+          int k = 0;
+#pragma unroll
+          for (int hb = 0; hb < 2; ++hb)
+            for (uint32_t m = mk[hb]; m && k < kRowCap;) {
+              const int e = __clz((int)m);
+              m &= ~(0x80000000u >> e);
+              cand[k++] = (uint8_t)((ch0 + hb) * 32 + e);
+            }
+        }
+      }
+      sCnt[qt * AT + row] = (int)word;
       named_bar_sync(1, AEW * 32);
       // the row owner (quarter 0) merges: one candidate decides, a few go to the pair list
       int best = 0;
       if (qt == 0) {
-        int c[4], tot = 0;
+        uint32_t cw[4];
+        int tot = 0;
         bool bad = false;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          c[q] = sCnt[q * AT + row];
-          bad = bad || c[q] < 0;
-          tot += c[q];
+          cw[q] = (uint32_t)sCnt[q * AT + row];
+          bad = bad || (cw[q] & 0xFFu) == 0xFFu;
+          tot += (int)(cw[q] & 0xFFu);
+          if (cw[q] & 0xFFu) best = (int)(cw[q] >> 8);
         }
         uint32_t rinfo = 0;
         if (bad || tot == 0 || tot > kRowCap) {
           rinfo = 0xFFFFu;  // every centroid, sequentially
-        } else if (tot == 1) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (c[q]) best = sCnd[(row * 4 + q) * kRowCap];
-        } else if (valid) {
+        } else if (tot > 1 && valid) {
           const int base = atomicAdd(s_np, tot);
           if (base + tot <= kPairCap) {
             int s2 = 0;
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-              for (int k = 0; k < c[q]; ++k)
-                sPJ[base + s2++] = ((uint32_t)row << 16) | (uint32_t)sCnd[(row * 4 + q) * kRowCap + k];
+            for (int q = 0; q < 4; ++q) {
+              const int n2 = (int)(cw[q] & 0xFFu);
+              for (int k = 0; k < n2; ++k)
+                sPJ[base + s2++] =
+                    ((uint32_t)row << 16) | (n2 == 1 ? cw[q] >> 8 : (uint32_t)sCnd[(row * 4 + q) * kRowCap + k]);
+            }
             rinfo = ((uint32_t)base << 16) | (uint32_t)tot;
           } else {
             rinfo = 0xFFFFu;
@@ -353,8 +417,8 @@ __global__ void __launch_bounds__(ANT, 1)
               best = (int)(sPJ[base + s2] & 0xFFFFu);
             }
         }
-        a.asg[(size_t)h * a.N + n] = (uint8_t)best;
-        atomicAdd(a.counts + (size_t)h * C + best, 1);
+        a.asg[(size_t)h * a.asg_stride + n] = (uint8_t)best;
+        if (!a.scan) atomicAdd(a.counts + (size_t)h * C + best, 1);
       }
       fence_proxy_async_smem();  // generic reads of tile b before the next copy into it
       tc_fence_before();
@@ -378,6 +442,8 @@ __global__ void __launch_bounds__(ANT, 1)
 // then each token to a slot of its cluster (any order within a cluster).
 __global__ void __launch_bounds__(1024) fit_scatter(const FitArgs a) {
   __shared__ int s_off[256], s_cur[256], s_wsum[8];
+  pdl_launch();
+  pdl_wait();
   const int h = blockIdx.x, tid = threadIdx.x, C = a.C, lane = tid & 31;
   // exclusive prefix of the counts over j (warp scans, then the warp totals)
   int v = 0, incl = 0;
@@ -391,7 +457,6 @@ __global__ void __launch_bounds__(1024) fit_scatter(const FitArgs a) {
     }
     if (lane == 31) s_wsum[tid >> 5] = incl;
   }
-  if (tid == 0) a.nmax[h] = 0u;  // rebuilt by fit_means
   __syncthreads();
   if (tid < 256) {
     int wp = 0;
@@ -404,7 +469,7 @@ __global__ void __launch_bounds__(1024) fit_scatter(const FitArgs a) {
     s_cur[tid] = 0;
   }
   __syncthreads();
-  const uint8_t* asg = a.asg + (size_t)h * a.N;
+  const uint8_t* asg = a.asg + (size_t)h * a.asg_stride;
   int32_t* lst = a.list + (size_t)h * a.N;
   // (the bounds checks only matter after a timed-out assignment left stale entries)
   for (int64_t n = tid; n < a.N; n += blockDim.x) {
@@ -420,6 +485,8 @@ __global__ void __launch_bounds__(1024) fit_scatter(const FitArgs a) {
 // 2^U of the exact fixed-point member sums (U = emax - 134 - room), and |x|^2
 // of every token, which sizes the screening bound.
 __global__ void __launch_bounds__(256) fit_scale(const FitArgs a) {
+  pdl_launch();
+  pdl_wait();
   const int h = blockIdx.y, lane = threadIdx.x & 31;
   uint32_t mx = 0;
   for (int64_t n = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); n < a.N; n += (int64_t)gridDim.x * 8) {
@@ -444,131 +511,212 @@ __global__ void __launch_bounds__(256) fit_scale(const FitArgs a) {
 //   integer (128 + f) << (e - 134 - U) < 2^(8 + room) in units of 2^U, and N
 //   of them add in int64 without overflow.  A member outside that grid (tiny,
 //   subnormal, inf or NaN) sends the cluster to fp64 sums instead.
-//   The mean RN32(RN64(S / n)): q = S * RN64(1/n) lies within 2.5 ulp of
-//   RN64(S / n), so both round to the same fp32 value unless q is within a
-//   few ulp of a point halfway between two fp32 values; there (and outside the
-//   fp32 normal range) the exact fp64 division decides.
-__device__ __forceinline__ float mean_of(int64_t k, int U, double invs, double dc, bool& exact_ok) {
-  const double kd = (double)k;
-  if (!((double)(kd) == (double)k && (long long)kd == k)) {
-    exact_ok = false;
-    return 0.0f;
-  }
-  const double q = kd * invs;
-  const long long bits = __double_as_longlong(q);
-  const int ex = (int)((bits >> 52) & 0x7FF);
-  const long long lo = bits & ((1LL << 29) - 1);
-  const bool near = (lo > (1LL << 28) - 16 && lo < (1LL << 28) + 16) || ex < 1023 - 126 || ex > 1023 + 127;
-  if (k != 0 && near) return __double2float_rn(__ddiv_rn(ldexp(kd, U), dc));
-  return __double2float_rn(q);
+//   The mean RN32(RN64(S / n)): S and 1 / n as pairs of fp32 values (S to 2^-48,
+//   1 / n to 2^-46 relative) and one product of pairs give S / n to 2^-44;
+//   its high part is the result unless the true quotient may lie within 2^-40
+//   relative of a point halfway between two fp32 values (which also covers the
+//   rounding to fp64 in between), or leaves the fp32 normal range: there the
+//   fp64 division decides.  (fp64 operations run at 1/64 of the fp32 rate.)
+__device__ __forceinline__ float mean_of(long long k, int U, float rh, float rl, double dc) {
+  const float kh = __ll2float_rn(k);
+  const float kl = __ll2float_rn(k - __float2ll_rn(kh));
+  const float ph = __fmul_rn(kh, rh);
+  const float pe = fmaf(kh, rl, fmaf(kl, rh, fmaf(kh, rh, -ph)));
+  const float q = __fadd_rn(ph, pe);
+  const float e = __fsub_rn(pe, __fsub_rn(q, ph));          // exact: |pe| is far below |ph|
+  const uint32_t qb = __float_as_uint(q) & 0x7FFFFFFFu;
+  const int ex = (int)(qb >> 23) + U;                        // exponent field of the mean
+  const float ulp = __uint_as_float((qb & 0x7F800000u) - (23u << 23));   // of q (|q| >= 2^-24: k is an integer)
+  // half an ulp, a quarter just below a power of two, less 2^-16 of it
+  const float lim = ulp * ((qb & 0x7FFFFFu) ? 0.49999237f : 0.24999619f);
+  if (k != 0 && (!(fabsf(e) < lim) || ex < 1 || ex > 254))
+    return __double2float_rn(__ddiv_rn(ldexp((double)k, U), dc));
+  return k == 0 ? 0.0f : __uint_as_float(__float_as_uint(q) + ((uint32_t)U << 23));
 }
 
-__global__ void __launch_bounds__(512) fit_means(const FitArgs a) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= (int64_t)a.H * a.C) return;
+// Four warps per centroid (the largest clusters hold many times the average,
+// and with one warp each they set the launch's time): the members go to the
+// warps in batches of eight rows; the warps' int64
+// sums meet in shared memory and warp 0 finishes.  Wan-14B Keys, per launch:
+// 51 us with a warp per centroid and a sorted list.
+__global__ void __launch_bounds__(128) fit_means(const FitArgs a, int last) {
+  __shared__ uint16_t s_list[kScanTokens];
+  __shared__ long long s_sum[4][128];
+  __shared__ int s_n, s_ok;
+  pdl_launch();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t w = blockIdx.x;
   const int h = (int)(w / a.C), j = (int)(w % a.C);
-  const int cnt = a.counts[w], base = a.offs[w];
-  float4* cr = reinterpret_cast<float4*>(a.cent + (size_t)w * 128) + lane;
-  float4 m;
-  if (cnt > 0) {
-    const int32_t* lst = a.list + (size_t)h * a.N + (base < a.N ? base : 0);
-    const int U = a.emax[h] - 134 - a.room;
-    int64_t k0 = 0, k1 = 0, k2 = 0, k3 = 0;
-    bool grid_ok = true;
-    // A member value in units of 2^U, y = (128 + f) 2^(e - 134 - U) < 2^48 (room <= 40),
-    // has 8 significant bits: the bf16 bits widened to fp32 with -U added to the
-    // exponent field.  Two additions of 3 2^54 and 3 2^38 split it exactly into
-    // fp32 limbs that are multiples of 2^32 and 2^16 and a remainder below
-    // 2^15; 32 such limbs add exactly in fp32 (below 2^21 units each), and every
-    // 32 members the three limb sums go to int64.  Zero stays zero; a value off
-    // the grid (tiny, subnormal, inf, NaN) clears grid_ok.
-    const uint32_t eadd = (uint32_t)(-U) << 23;
-    const int emin = U + 134;
-    const float C32 = 5.4043195528445952e16f;   // 3 * 2^54
-    const float C16 = 8.24633720832e11f;        // 3 * 2^38
-    float l2[4], l1[4], l0[4];
-    auto limb = [&](uint32_t b16, int ch) {
-      const uint32_t e = (b16 >> 7) & 0xFFu;
-      const bool zero = (b16 & 0x7FFFu) == 0u;
-      grid_ok = grid_ok && (zero || ((int)e >= emin && e != 255u));
-      const float y = zero ? 0.0f : __uint_as_float((b16 << 16) + eadd);
-      const float hi = __fsub_rn(__fadd_rn(y, C32), C32);
-      const float r1 = __fsub_rn(y, hi);
-      const float mid = __fsub_rn(__fadd_rn(r1, C16), C16);
-      l2[ch] = __fadd_rn(l2[ch], hi);
-      l1[ch] = __fadd_rn(l1[ch], mid);
-      l0[ch] = __fadd_rn(l0[ch], __fsub_rn(r1, mid));
-    };
-    auto flush = [&](int64_t& k, int ch) {
-      k += ((int64_t)__float2int_rn(l2[ch] * 2.3283064365386963e-10f) << 32) +
-           ((int64_t)__float2int_rn(l1[ch] * 1.52587890625e-05f) << 16) + (int64_t)__float2int_rn(l0[ch]);
-    };
-    for (int i0 = 0; i0 < cnt; i0 += 32) {
-      const int nb = min(32, cnt - i0);
-      const int my = lane < nb ? lst[i0 + lane] : -1;  // 32 member indices in one read
+  if (tid == 0) {
+    s_n = 0;
+    s_ok = 1;
+  }
+  __syncthreads();
+  pdl_wait();
+  const uint8_t* asg = a.asg + (size_t)h * a.asg_stride;
+  const int U = a.emax[h] - 134 - a.room;
+  int64_t k0 = 0, k1 = 0, k2 = 0, k3 = 0;
+  bool grid_ok = true;
+  // A member value in units of 2^U, y = (128 + f) 2^(e - 134 - U) < 2^48 (room <= 40),
+  // has 8 significant bits: the bf16 bits widened to fp32 with -U added to the
+  // exponent field.  Two additions of 3 2^54 and 3 2^38 split it exactly into
+  // fp32 limbs that are multiples of 2^32 and 2^16 and a remainder below
+  // 2^15; 32 such limbs add exactly in fp32 (below 2^21 units each), and every
+  // 32 members the three limb sums go to int64.  Zero stays zero; a value off
+  // the grid (tiny, subnormal, inf, NaN) clears grid_ok.
+  const uint32_t eadd = (uint32_t)(-U) << 23;
+  const int emin = U + 134;
+  const float C32 = 5.4043195528445952e16f;   // 3 * 2^54
+  const float C16 = 8.24633720832e11f;        // 3 * 2^38
+  float l2[4] = {}, l1[4] = {}, l0[4] = {};
+  auto limb = [&](uint32_t b16, int ch) {
+    const uint32_t e = (b16 >> 7) & 0xFFu;
+    const bool zero = (b16 & 0x7FFFu) == 0u;
+    grid_ok = grid_ok && (zero || ((int)e >= emin && e != 255u));
+    const float y = zero ? 0.0f : __uint_as_float((b16 << 16) + eadd);
+    const float hi = __fsub_rn(__fadd_rn(y, C32), C32);
+    const float r1 = __fsub_rn(y, hi);
+    const float mid = __fsub_rn(__fadd_rn(r1, C16), C16);
+    l2[ch] = __fadd_rn(l2[ch], hi);
+    l1[ch] = __fadd_rn(l1[ch], mid);
+    l0[ch] = __fadd_rn(l0[ch], __fsub_rn(r1, mid));
+  };
+  auto flush = [&](int64_t& k, int ch) {
+    k += ((int64_t)__float2int_rn(l2[ch] * 2.3283064365386963e-10f) << 32) +
+         ((int64_t)__float2int_rn(l1[ch] * 1.52587890625e-05f) << 16) + (int64_t)__float2int_rn(l0[ch]);
+    l2[ch] = l1[ch] = l0[ch] = 0.0f;
+  };
+  int since = 0;   // members since the last flush
+  // the rows of batches warp, warp + 4, ... of n members, token(m) the m-th
+  auto rows = [&](int n, auto token) {
+    for (int b = 8 * warp; b < n; b += 32) {
+      uint2 xv[8];
 #pragma unroll
-      for (int ch = 0; ch < 4; ++ch) l2[ch] = l1[ch] = l0[ch] = 0.0f;
-      for (int kb = 0; kb < nb; kb += 8) {
-        uint2 xv[8];
+      for (int k = 0; k < 8; ++k) {
+        xv[k] = make_uint2(0, 0);
+        const int64_t tok = b + k < n ? token(b + k) : -1;
+        if (tok >= 0 && tok < a.N)  // always a token, unless a timed-out assignment left stale entries
+          xv[k] = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
+      }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int tok = __shfl_sync(0xFFFFFFFFu, my, (kb + k) & 31);
-          xv[k] = make_uint2(0, 0);
-          if (kb + k < nb && tok >= 0 && tok < a.N)  // always, unless a timed-out assignment left stale lists
-            xv[k] = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
-        }
+      for (int k = 0; k < 8; ++k) {
+        limb(xv[k].x & 0xFFFFu, 0);
+        limb(xv[k].x >> 16, 1);
+        limb(xv[k].y & 0xFFFFu, 2);
+        limb(xv[k].y >> 16, 3);
+      }
+      if ((since += 8) == 32) {
+        since = 0;
+        flush(k0, 0);
+        flush(k1, 1);
+        flush(k2, 2);
+        flush(k3, 3);
+      }
+    }
+  };
+  int cnt = 0;
+  if (a.scan) {
+    const uint32_t jj = (uint32_t)j * 0x01010101u;
+    for (int o = 16 * tid; o < a.N; o += 16 * 128) {
+      const uint4 v = *reinterpret_cast<const uint4*>(asg + o);   // rows are padded to 16 bytes
+      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          limb(xv[k].x & 0xFFFFu, 0);
-          limb(xv[k].x >> 16, 1);
-          limb(xv[k].y & 0xFFFFu, 2);
-          limb(xv[k].y >> 16, 3);
+      for (int q = 0; q < 4; ++q) {
+        uint32_t m = __vcmpeq4(w4[q], jj) & 0x01010101u;
+        while (m) {
+          const int t = o + 4 * q + ((__ffs((int)m) - 1) >> 3);
+          m &= m - 1;
+          if (t < a.N) s_list[atomicAdd(&s_n, 1)] = (uint16_t)t;
         }
       }
-      flush(k0, 0);
-      flush(k1, 1);
-      flush(k2, 2);
-      flush(k3, 3);
     }
+    __syncthreads();
+    cnt = s_n;
+    rows(cnt, [&](int m) { return (int64_t)s_list[m]; });
+  } else {
+    cnt = a.counts[w];
+    const int base = a.offs[w];
+    const int32_t* lst = a.list + (size_t)h * a.N + (base < a.N ? base : 0);
+    rows(cnt, [&](int m) { return (int64_t)lst[m]; });
+  }
+  flush(k0, 0);
+  flush(k1, 1);
+  flush(k2, 2);
+  flush(k3, 3);
+  s_sum[warp][4 * lane] = k0;
+  s_sum[warp][4 * lane + 1] = k1;
+  s_sum[warp][4 * lane + 2] = k2;
+  s_sum[warp][4 * lane + 3] = k3;
+  if (!grid_ok) s_ok = 0;
+  __syncthreads();
+  if (warp != 0) return;
+
+  float4* cr = reinterpret_cast<float4*>(a.cent + (size_t)w * 128) + lane;
+  float4 m = *cr;
+  if (cnt > 0) {
     const double dc = (double)cnt;
-    bool ok = __all_sync(0xFFFFFFFFu, grid_ok);
+    bool ok = s_ok != 0 && cnt <= (1 << 24);
     if (ok) {
-      const double invs = ldexp(__ddiv_rn(1.0, dc), U);
-      bool eo = true;
-      m = make_float4(mean_of(k0, U, invs, dc, eo), mean_of(k1, U, invs, dc, eo), mean_of(k2, U, invs, dc, eo),
-                      mean_of(k3, U, invs, dc, eo));
-      ok = __all_sync(0xFFFFFFFFu, eo);
+      auto total = [&](int ch) {
+        return s_sum[0][4 * lane + ch] + s_sum[1][4 * lane + ch] + s_sum[2][4 * lane + ch] + s_sum[3][4 * lane + ch];
+      };
+      const float n = (float)cnt;   // exact: cnt <= 2^24
+      const float rh = __frcp_rn(n), rl = __fmul_rn(fmaf(-n, rh, 1.0f), rh);
+      bool rep = true;   // every sum exact in fp64, as the definition's is
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch) {
+        const long long t = total(ch);
+        rep = rep && ((t < (1LL << 53) && t > -(1LL << 53)) || (long long)(double)t == t);
+      }
+      ok = __all_sync(0xFFFFFFFFu, rep);
+      if (ok)
+        m = make_float4(mean_of(total(0), U, rh, rl, dc), mean_of(total(1), U, rh, rl, dc),
+                        mean_of(total(2), U, rh, rl, dc), mean_of(total(3), U, rh, rl, dc));
     }
     if (!ok) {  // fp64 sums (exact for members of ordinary range)
       double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      for (int i = 0; i < cnt; ++i) {
-        const int64_t tok = lst[i];
-        if (tok < 0 || tok >= a.N) continue;
+      auto add = [&](int64_t tok) {
         const uint2 xv = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
         s0 += (double)__uint_as_float(xv.x << 16);
         s1 += (double)__uint_as_float(xv.x & 0xFFFF0000u);
         s2 += (double)__uint_as_float(xv.y << 16);
         s3 += (double)__uint_as_float(xv.y & 0xFFFF0000u);
+      };
+      if (a.scan) {
+        for (int64_t n0 = 0; n0 < a.N; n0 += 32) {
+          uint32_t mk = __ballot_sync(0xFFFFFFFFu, n0 + lane < a.N && asg[n0 + lane] == (uint8_t)j);
+          for (; mk; mk &= mk - 1) add(n0 + __ffs((int)mk) - 1);
+        }
+      } else {
+        const int base = a.offs[w];
+        const int32_t* lst = a.list + (size_t)h * a.N + (base < a.N ? base : 0);
+        for (int i = 0; i < cnt; ++i) {
+          const int64_t tok = lst[i];
+          if (tok >= 0 && tok < a.N) add(tok);
+        }
       }
       m = make_float4(__double2float_rn(__ddiv_rn(s0, dc)), __double2float_rn(__ddiv_rn(s1, dc)),
                       __double2float_rn(__ddiv_rn(s2, dc)), __double2float_rn(__ddiv_rn(s3, dc)));
     }
     *cr = m;
-  } else {
-    m = *cr;
+  }
+  if (last) {
+    // the bf16 result; NaN everywhere if a wait inside an assignment ran out
+    const bool bad = *a.status != 0;
+    const uint32_t nan2 = 0x7FFF7FFFu;
+    reinterpret_cast<uint2*>(a.out + (size_t)w * 128)[lane] =
+        bad ? make_uint2(nan2, nan2) : make_uint2(pack_bf16(m.x, m.y), pack_bf16(m.z, m.w));
+    return;
   }
   emit_row(a, h, j, m, lane);
-  __syncwarp();
-  if (lane == 0) a.counts[w] = 0;  // ready for the next assignment
+  if (lane == 0 && !a.scan) a.counts[w] = 0;  // ready for the next assignment
 }
 
-// bf16 output; NaN everywhere if a wait inside the assignment ran out.
+// bf16 output of the initial centroids (no iteration).
 __global__ void fit_out(const FitArgs a) {
   const int64_t n = (int64_t)a.H * a.C * 128;
-  const bool bad = *a.status != 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    a.out[i] = bad ? __float2bfloat16_rn(NAN) : __float2bfloat16_rn(a.cent[i]);
+    a.out[i] = __float2bfloat16_rn(a.cent[i]);
 }
 
 int sm_count() {
@@ -589,7 +737,7 @@ size_t fit_workspace_bytes(int H, int d, int C, int64_t N) {
   b += (size_t)round_up((int64_t)H * C * d * 4, 256);           // cent
   b += (size_t)round_up((int64_t)H * Np * 512, 256);            // images
   b += (size_t)round_up((int64_t)H * Np * 4, 256);              // norms
-  b += 2 * (size_t)round_up((int64_t)H * 4, 256);               // largest norm, largest exponent
+  b += 2 * (size_t)round_up((int64_t)H * 4, 256);               // largest exponent (and a reserved field)
   b += 2 * (size_t)round_up((int64_t)H * C * 4, 256);           // counts, offsets
   b += (size_t)round_up((int64_t)H * N, 256);                   // assignment
   b += (size_t)round_up((int64_t)H * N * 4, 256);               // token norms
@@ -608,8 +756,8 @@ void fit_carve(FitArgs& a, uint8_t* ws) {
   a.status = reinterpret_cast<int32_t*>(take(256));
   a.cent = reinterpret_cast<float*>(take((int64_t)a.H * a.C * a.d * 4));
   a.img = take((int64_t)a.H * a.Npad * 512);
-  a.nrm = reinterpret_cast<float*>(take((int64_t)a.H * a.Npad * 4));
-  a.nmax = reinterpret_cast<uint32_t*>(take((int64_t)a.H * 4));
+  a.nrm = reinterpret_cast<uint32_t*>(take((int64_t)a.H * a.Npad * 4));
+  take((int64_t)a.H * 4);   // reserved
   a.emax = reinterpret_cast<int32_t*>(take((int64_t)a.H * 4));
   // member sums of at most N values below 2^(8 + room) each stay below 2^61, and
   // each value below 2^48 units
@@ -621,37 +769,59 @@ void fit_carve(FitArgs& a, uint8_t* ws) {
   a.asg = take((int64_t)a.H * a.N);
   a.xn2 = reinterpret_cast<float*>(take((int64_t)a.H * a.N * 4));
   a.list = reinterpret_cast<int32_t*>(take((int64_t)a.H * a.N * 4));
+  // Up to kScanTokens tokens the means pick their members out of the assignment
+  // bytes (every centroid of a head reads them all: at 8192 tokens as much as
+  // the rows of the members), which then lie in the list's place, each head's
+  // padded to 16 bytes; beyond that the sorted list is built.
+  a.scan = a.N >= 16 && a.N <= kScanTokens;
+  a.asg_stride = a.scan ? round_up(a.N, 16) : a.N;
+  if (a.scan) a.asg = reinterpret_cast<uint8_t*>(a.list);
 }
+
+namespace {
+// A launch that may start its prologue before the one in front of it has ended.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = grid;
+  lc.blockDim = dim3((unsigned)threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, k, static_cast<P>(args)...);
+}
+}  // namespace
 
 cudaError_t launch_fit(const FitArgs& a, cudaStream_t st) {
   cudaError_t e;
-  if ((e = cudaMemsetAsync(a.status, 0, 4, st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(a.nmax, 0, (size_t)a.H * 4, st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(a.emax, 0, (size_t)a.H * 4, st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(a.counts, 0, (size_t)a.H * a.C * 4, st)) != cudaSuccess) return e;
   const int64_t prep_warps = (int64_t)a.H * a.Npad;
   fit_prep<<<(unsigned)((prep_warps + 15) / 16), 512, 0, st>>>(a);
-  if (a.iters > 0) {
-    CUtensorMap tm;
-    if (!make_token_map(&tm, a.x, a.N, a.H, 128)) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(fit_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM)) != cudaSuccess)
-      return e;
-    const int tiles = (int)((a.N + 127) / 128);
-    const int units = a.H * tiles;
-    const int grid = units < sm_count() ? units : sm_count();
-    const int64_t mean_warps = (int64_t)a.H * a.C;
-    const int64_t sb = (a.N + 7) / 8;
-    fit_scale<<<dim3((unsigned)(sb < 64 ? sb : 64), (unsigned)a.H), 256, 0, st>>>(a);
-    for (int it = 0; it < a.iters; ++it) {
-      fit_assign<<<grid, ANT, A_SMEM, st>>>(a, tm, tiles, units);
-      fit_scatter<<<a.H, 1024, 0, st>>>(a);
-      fit_means<<<(unsigned)((mean_warps + 15) / 16), 512, 0, st>>>(a);
-    }
+  if (a.iters == 0) {
+    const int64_t n = (int64_t)a.H * a.C * a.d;
+    fit_out<<<(unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, st>>>(a);
+    return cudaGetLastError();
   }
-  const int64_t n = (int64_t)a.H * a.C * a.d;
-  const unsigned og = (unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  fit_out<<<og, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  CUtensorMap tm;
+  if (!make_token_map(&tm, a.x, a.N, a.H, 128)) return cudaErrorInvalidValue;
+  if ((e = cudaFuncSetAttribute(fit_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM)) != cudaSuccess)
+    return e;
+  const int tiles = (int)((a.N + 127) / 128);
+  const int units = a.H * tiles;
+  const int sms = sm_count();
+  const int grid = units < sms ? units : sms;
+  const int64_t sb = (a.N + 7) / 8;
+  e = launch_pdl(fit_scale, dim3((unsigned)(sb < 64 ? sb : 64), (unsigned)a.H), 256, 0, st, a);
+  for (int it = 0; it < a.iters && e == cudaSuccess; ++it) {
+    e = launch_pdl(fit_assign, dim3((unsigned)grid), ANT, A_SMEM, st, a, tm, tiles, units);
+    if (e == cudaSuccess && !a.scan) e = launch_pdl(fit_scatter, dim3((unsigned)a.H), 1024, 0, st, a);
+    if (e == cudaSuccess)
+      e = launch_pdl(fit_means, dim3((unsigned)((int64_t)a.H * a.C)), 128, 0, st, a, (int)(it + 1 == a.iters));
+  }
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 }  // namespace qwm

@@ -346,6 +346,26 @@ __device__ __forceinline__ float tmem_ld128_max(uint32_t t, float (&v)[128]) {
   return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
 }
 
+// 32 + 32 columns (at ta and tb) of each thread's lane with their maximum: two
+// reducing loads and one wait.
+__device__ __forceinline__ float tmem_ld64_max(uint32_t ta, uint32_t tb, float (&v)[64]) {
+  uint32_t r[64];
+  float m[2];
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+    asm volatile(
+        "tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, %32, [%33];"
+        : "=r"(r[32 * b + 0]), "=r"(r[32 * b + 1]), "=r"(r[32 * b + 2]), "=r"(r[32 * b + 3]), "=r"(r[32 * b + 4]), "=r"(r[32 * b + 5]), "=r"(r[32 * b + 6]), "=r"(r[32 * b + 7]), "=r"(r[32 * b + 8]), "=r"(r[32 * b + 9]), "=r"(r[32 * b + 10]), "=r"(r[32 * b + 11]), "=r"(r[32 * b + 12]), "=r"(r[32 * b + 13]), "=r"(r[32 * b + 14]), "=r"(r[32 * b + 15]), "=r"(r[32 * b + 16]), "=r"(r[32 * b + 17]), "=r"(r[32 * b + 18]), "=r"(r[32 * b + 19]), "=r"(r[32 * b + 20]), "=r"(r[32 * b + 21]), "=r"(r[32 * b + 22]), "=r"(r[32 * b + 23]), "=r"(r[32 * b + 24]), "=r"(r[32 * b + 25]), "=r"(r[32 * b + 26]), "=r"(r[32 * b + 27]), "=r"(r[32 * b + 28]), "=r"(r[32 * b + 29]), "=r"(r[32 * b + 30]), "=r"(r[32 * b + 31]), "=f"(m[b])
+        : "r"(b ? tb : ta));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]), "+r"(r[32]), "+r"(r[33]), "+r"(r[34]), "+r"(r[35]), "+r"(r[36]), "+r"(r[37]), "+r"(r[38]), "+r"(r[39]), "+r"(r[40]), "+r"(r[41]), "+r"(r[42]), "+r"(r[43]), "+r"(r[44]), "+r"(r[45]), "+r"(r[46]), "+r"(r[47]), "+r"(r[48]), "+r"(r[49]), "+r"(r[50]), "+r"(r[51]), "+r"(r[52]), "+r"(r[53]), "+r"(r[54]), "+r"(r[55]), "+r"(r[56]), "+r"(r[57]), "+r"(r[58]), "+r"(r[59]), "+r"(r[60]), "+r"(r[61]), "+r"(r[62]), "+r"(r[63]), "+f"(m[0]), "+f"(m[1])
+               :
+               : "memory");
+#pragma unroll
+  for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+  return fmaxf(m[0], m[1]);
+}
+
 // 32 lanes x 32 consecutive 32-bit columns (not waited for).
 __device__ __forceinline__ void tmem_st32u(uint32_t taddr, const uint32_t* v) {
   asm volatile(

@@ -216,14 +216,15 @@ struct FitArgs {
   int32_t* status;             // device status word (a bounded wait that ran out)
   float* cent;                 // [H][C][d] fp32 centroids
   uint8_t* img;                // [H][2][Npad * 256] bf16 MMA operand images: hi, lo
-  float* nrm;                  // [H][Npad] squared centroid norms
-  uint32_t* nmax;              // [H] largest squared norm (fp32 bits)
+  uint32_t* nrm;               // [H][Npad] minus half the squared centroid norms, two bf16 parts
   int32_t* emax;               // [H] largest bf16 exponent field of the head's tokens
   float* xn2;                  // [H][N] |x|^2 of every token (fp32, any order)
   int room;                    // fixed-point headroom bits of the exact member sums
   int32_t* counts;             // [H][C] members per cluster
   int32_t* offs;               // [H][C] first member slot
-  uint8_t* asg;                // [H][N] assignment
+  bool scan;                   // the means scan the assignment instead of reading the sorted list
+  int64_t asg_stride;
+  uint8_t* asg;                // [H][asg_stride] assignment
   int32_t* list;               // [H][N] member token indices grouped by cluster
 };
 struct DequantArgs {
