@@ -27,12 +27,11 @@
 //     s_j > s_k - c (|x|^2 + 2.02 (|x|^2 + d)) is a candidate for the exact
 //     argmin.  A row with a single candidate is decided, the others are
 //     rescored with the sequential fp32 distance.
-//   fit_means   (four warps per centroid): the members of a centroid are picked
-//     out of the head's assignment bytes (more than kScanTokens tokens: read
-//     from a list that fit_scatter, one CTA per head, sorts by cluster); exact
-//     member sums (bf16 values of ordinary range add exactly, so the order does
-//     not matter), the mean, and the next iteration's operand images and norm;
-//     the last iteration's launch writes the bf16 result.
+//   fit_means   (four warps per centroid): exact member sums (bf16 values of
+//     ordinary range add exactly, so the order does not matter) from the list of
+//     members that the assignment leaves per centroid, the mean, and the next
+//     iteration's operand images and norm; the last iteration's launch writes the
+//     bf16 result.
 // Each launch is a programmatic dependent of the one before it (its prologue
 // overlaps that one's tail).
 #include <mutex>
@@ -45,7 +44,6 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kScanTokens = 8192;             // tokens up to which fit_means scans the assignment (fit_carve)
 constexpr int AT = 128;                       // tokens per tile
 constexpr int AEW = 16;                       // epilogue warps: rows 32 (w & 3) + lane, column quarter w >> 2
 constexpr int ANT = (AEW + 1) * 32;           // + one producer / MMA warp
@@ -93,19 +91,23 @@ __device__ __forceinline__ int sw_off(int rows, int row, int ch) {
 }
 
 // The sequential fp32 distance of the definition: channel order, the
-// difference, its square and the running sum each rounded on its own.  The
-// centroid row is fetched whole first (one memory round trip), then summed.
+// difference, its square and the running sum each rounded on its own.
 __device__ float exact_dist(const uint8_t* sX, int row, const float* mu) {
-  float4 mv[32];
+  const float4* m4 = reinterpret_cast<const float4*>(mu);
+  float4 mv[16];   // a ring of 64 channels: the loads run ahead of the chain
 #pragma unroll
-  for (int i = 0; i < 32; ++i) mv[i] = __ldg(reinterpret_cast<const float4*>(mu) + i);
+  for (int i = 0; i < 16; ++i) mv[i] = __ldg(m4 + i);
   float acc = 0.0f;
 #pragma unroll
   for (int ch = 0; ch < 16; ++ch) {
     const uint4 xv = *reinterpret_cast<const uint4*>(sX + sw_off(128, row, ch));
     const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
-    const float ms[8] = {mv[2 * ch].x, mv[2 * ch].y, mv[2 * ch].z, mv[2 * ch].w,
-                         mv[2 * ch + 1].x, mv[2 * ch + 1].y, mv[2 * ch + 1].z, mv[2 * ch + 1].w};
+    const float4 ma = mv[(2 * ch) & 15], mb = mv[(2 * ch + 1) & 15];
+    if (ch < 8) {
+      mv[2 * ch] = __ldg(m4 + 2 * ch + 16);
+      mv[2 * ch + 1] = __ldg(m4 + 2 * ch + 17);
+    }
+    const float ms[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const float xe = (e & 1) ? __uint_as_float(xw[e >> 1] & 0xFFFF0000u) : __uint_as_float(xw[e >> 1] << 16);
@@ -299,6 +301,16 @@ __global__ void __launch_bounds__(ANT, 1)
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
     const int nchunk = (Npad + 31) >> 5;
     const int ch0 = (qt * nchunk) >> 2, ch1 = ((qt + 1) * nchunk) >> 2;   // this quarter's 32-column chunks
+    // A token's place among its centroid's members comes back from an atomic
+    // count; it is listed one tile later, when that has long arrived.
+    int pl_rank = 0, pl_tok = -1;
+    size_t pl_cent = 0;
+    auto list_member = [&]() {
+      if (pl_tok < 0 || pl_rank >= a.cap) return;
+      const size_t at = pl_cent * a.cap + pl_rank;
+      if (a.wide) reinterpret_cast<int32_t*>(a.list)[at] = pl_tok;
+      else reinterpret_cast<uint16_t*>(a.list)[at] = (uint16_t)pl_tok;
+    };
     for (int t = 0; t < T; ++t) {
       const int u = u0 + t, h = u / tiles, tile = u - h * tiles, b = t & 1;
       const uint8_t* sX = sm + A_X + b * 32768;
@@ -417,8 +429,11 @@ __global__ void __launch_bounds__(ANT, 1)
               best = (int)(sPJ[base + s2] & 0xFFFFu);
             }
         }
-        a.asg[(size_t)h * a.asg_stride + n] = (uint8_t)best;
-        if (!a.scan) atomicAdd(a.counts + (size_t)h * C + best, 1);
+        a.asg[(size_t)h * a.N + n] = (uint8_t)best;
+        list_member();
+        pl_cent = (size_t)h * C + best;
+        pl_tok = (int)n;
+        pl_rank = atomicAdd(a.counts + pl_cent, 1);
       }
       fence_proxy_async_smem();  // generic reads of tile b before the next copy into it
       tc_fence_before();
@@ -428,6 +443,7 @@ __global__ void __launch_bounds__(ANT, 1)
       if (lane == 0) mbar_arrive(bar_free(b));
       if (!go) break;
     }
+    if (qt == 0) list_member();
   }
   if (tid == 0 && *s_err) atomicCAS(a.status, 0, (int)QWM_ERR_TIMEOUT);
   tc_fence_before();
@@ -435,49 +451,6 @@ __global__ void __launch_bounds__(ANT, 1)
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tbase, 2 * ncols);
-  }
-}
-
-// Counting sort of one head's tokens by cluster: offsets from the counts,
-// then each token to a slot of its cluster (any order within a cluster).
-__global__ void __launch_bounds__(1024) fit_scatter(const FitArgs a) {
-  __shared__ int s_off[256], s_cur[256], s_wsum[8];
-  pdl_launch();
-  pdl_wait();
-  const int h = blockIdx.x, tid = threadIdx.x, C = a.C, lane = tid & 31;
-  // exclusive prefix of the counts over j (warp scans, then the warp totals)
-  int v = 0, incl = 0;
-  if (tid < 256) {
-    v = tid < C ? a.counts[(size_t)h * C + tid] : 0;
-    incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_wsum[tid >> 5] = incl;
-  }
-  __syncthreads();
-  if (tid < 256) {
-    int wp = 0;
-    for (int k = 0; k < (tid >> 5); ++k) wp += s_wsum[k];
-    s_off[tid] = wp + incl - v;
-  }
-  __syncthreads();
-  if (tid < C) {
-    a.offs[(size_t)h * C + tid] = s_off[tid];
-    s_cur[tid] = 0;
-  }
-  __syncthreads();
-  const uint8_t* asg = a.asg + (size_t)h * a.asg_stride;
-  int32_t* lst = a.list + (size_t)h * a.N;
-  // (the bounds checks only matter after a timed-out assignment left stale entries)
-  for (int64_t n = tid; n < a.N; n += blockDim.x) {
-    const int j = asg[n];
-    if (j < C) {
-      const int pos = s_off[j] + atomicAdd(&s_cur[j], 1);
-      if (pos < a.N) lst[pos] = (int32_t)n;
-    }
   }
 }
 
@@ -535,12 +508,14 @@ __device__ __forceinline__ float mean_of(long long k, int U, float rh, float rl,
 }
 
 // Four warps per centroid (the largest clusters hold many times the average,
-// and with one warp each they set the launch's time): the members go to the
-// warps in batches of eight rows; the warps' int64
-// sums meet in shared memory and warp 0 finishes.  Wan-14B Keys, per launch:
-// 51 us with a warp per centroid and a sorted list.
+// and with one warp each they set the launch's time): batches of eight members
+// go round the warps, whose int64 sums meet in shared memory; warp 0 finishes.
+// The members are the centroid's list where the assignment had room for all of
+// them (twice the average cluster), else they are picked out of the head's
+// assignment bytes, kPick tokens at a time.
+constexpr int kPick = 4096;
 __global__ void __launch_bounds__(128) fit_means(const FitArgs a, int last) {
-  __shared__ uint16_t s_list[kScanTokens];
+  __shared__ uint16_t s_list[kPick];
   __shared__ long long s_sum[4][128];
   __shared__ int s_n, s_ok;
   pdl_launch();
@@ -551,29 +526,28 @@ __global__ void __launch_bounds__(128) fit_means(const FitArgs a, int last) {
     s_n = 0;
     s_ok = 1;
   }
-  __syncthreads();
   pdl_wait();
-  const uint8_t* asg = a.asg + (size_t)h * a.asg_stride;
+  const int cnt = a.counts[w];
   const int U = a.emax[h] - 134 - a.room;
-  int64_t k0 = 0, k1 = 0, k2 = 0, k3 = 0;
-  bool grid_ok = true;
-  // A member value in units of 2^U, y = (128 + f) 2^(e - 134 - U) < 2^48 (room <= 40),
-  // has 8 significant bits: the bf16 bits widened to fp32 with -U added to the
-  // exponent field.  Two additions of 3 2^54 and 3 2^38 split it exactly into
-  // fp32 limbs that are multiples of 2^32 and 2^16 and a remainder below
-  // 2^15; 32 such limbs add exactly in fp32 (below 2^21 units each), and every
-  // 32 members the three limb sums go to int64.  Zero stays zero; a value off
-  // the grid (tiny, subnormal, inf, NaN) clears grid_ok.
-  const uint32_t eadd = (uint32_t)(-U) << 23;
-  const int emin = U + 134;
+  float4* cr = reinterpret_cast<float4*>(a.cent + (size_t)w * 128) + lane;
+  float4 m = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (warp == 0) m = *cr;
+  __syncthreads();
+  // Exact member sums.  A member value in units of 2^U, y = (128 + f) 2^(e - 134
+  // - U) < 2^48 (room <= 40), has 8 significant bits.  Two additions of 3 2^54
+  // and 3 2^38 split it exactly into fp32 limbs that are multiples of 2^32 and
+  // 2^16 and a remainder below 2^15; 32 such limbs add exactly in fp32 (below
+  // 2^21 units each), and every 32 members the three limb sums go to int64.  A
+  // value off the grid (tiny, subnormal, inf, NaN) or a unit beyond the fp32
+  // range sends the cluster to fp64 sums.
+  const float unit = U >= -127 ? __uint_as_float((uint32_t)(127 - U) << 23) : 0.0f;   // 2^-U
   const float C32 = 5.4043195528445952e16f;   // 3 * 2^54
   const float C16 = 8.24633720832e11f;        // 3 * 2^38
+  int64_t k0 = 0, k1 = 0, k2 = 0, k3 = 0;
+  uint32_t least = 0xFFFFFFFFu, most = 0u;    // smallest magnitude - 1 (zero wraps) and largest, of bf16 pairs
   float l2[4] = {}, l1[4] = {}, l0[4] = {};
-  auto limb = [&](uint32_t b16, int ch) {
-    const uint32_t e = (b16 >> 7) & 0xFFu;
-    const bool zero = (b16 & 0x7FFFu) == 0u;
-    grid_ok = grid_ok && (zero || ((int)e >= emin && e != 255u));
-    const float y = zero ? 0.0f : __uint_as_float((b16 << 16) + eadd);
+  auto limb = [&](float x, int ch) {
+    const float y = __fmul_rn(x, unit);
     const float hi = __fsub_rn(__fadd_rn(y, C32), C32);
     const float r1 = __fsub_rn(y, hi);
     const float mid = __fsub_rn(__fadd_rn(r1, C16), C16);
@@ -581,78 +555,94 @@ __global__ void __launch_bounds__(128) fit_means(const FitArgs a, int last) {
     l1[ch] = __fadd_rn(l1[ch], mid);
     l0[ch] = __fadd_rn(l0[ch], __fsub_rn(r1, mid));
   };
+  auto pair = [&](uint32_t v, int ch) {
+    const uint32_t mag = v & 0x7FFF7FFFu;
+    least = vmin_u16x2(least, vadd_u16x2(mag, 0xFFFFFFFFu));
+    most = vmax_u16x2(most, mag);
+    limb(__uint_as_float(v << 16), ch);
+    limb(__uint_as_float(v & 0xFFFF0000u), ch + 1);
+  };
   auto flush = [&](int64_t& k, int ch) {
     k += ((int64_t)__float2int_rn(l2[ch] * 2.3283064365386963e-10f) << 32) +
          ((int64_t)__float2int_rn(l1[ch] * 1.52587890625e-05f) << 16) + (int64_t)__float2int_rn(l0[ch]);
     l2[ch] = l1[ch] = l0[ch] = 0.0f;
   };
-  int since = 0;   // members since the last flush
-  // the rows of batches warp, warp + 4, ... of n members, token(m) the m-th
-  auto rows = [&](int n, auto token) {
-    for (int b = 8 * warp; b < n; b += 32) {
-      uint2 xv[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        xv[k] = make_uint2(0, 0);
-        const int64_t tok = b + k < n ? token(b + k) : -1;
-        if (tok >= 0 && tok < a.N)  // always a token, unless a timed-out assignment left stale entries
-          xv[k] = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        limb(xv[k].x & 0xFFFFu, 0);
-        limb(xv[k].x >> 16, 1);
-        limb(xv[k].y & 0xFFFFu, 2);
-        limb(xv[k].y >> 16, 3);
-      }
-      if ((since += 8) == 32) {
-        since = 0;
-        flush(k0, 0);
-        flush(k1, 1);
-        flush(k2, 2);
-        flush(k3, 3);
-      }
-    }
+  auto flush_all = [&]() {
+    flush(k0, 0);
+    flush(k1, 1);
+    flush(k2, 2);
+    flush(k3, 3);
   };
-  int cnt = 0;
-  if (a.scan) {
-    const uint32_t jj = (uint32_t)j * 0x01010101u;
-    for (int o = 16 * tid; o < a.N; o += 16 * 128) {
-      const uint4 v = *reinterpret_cast<const uint4*>(asg + o);   // rows are padded to 16 bytes
-      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+  // batches warp, warp + 4, ... of n members, token(m) the m-th: lane 8 i + k
+  // reads the token of row k of the i-th of four batches
+  auto rows = [&](int n, auto token) {
+    for (int b0 = 8 * warp; b0 < n; b0 += 128) {
+      const int mine = b0 + 32 * (lane >> 3) + (lane & 7);
+      const int64_t tk = mine < n ? token(mine) : -1;
+#pragma unroll 1
+      for (int i = 0; i < 4 && b0 + 32 * i < n; ++i) {
+        uint2 xv[8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t m = __vcmpeq4(w4[q], jj) & 0x01010101u;
-        while (m) {
-          const int t = o + 4 * q + ((__ffs((int)m) - 1) >> 3);
-          m &= m - 1;
-          if (t < a.N) s_list[atomicAdd(&s_n, 1)] = (uint16_t)t;
+        for (int k = 0; k < 8; ++k) {
+          const int64_t tok = __shfl_sync(0xFFFFFFFFu, tk, 8 * i + k);
+          xv[k] = make_uint2(0, 0);
+          if (tok >= 0 && tok < a.N)  // every member, unless a timed-out assignment left stale entries
+            xv[k] = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          pair(xv[k].x, 0);
+          pair(xv[k].y, 2);
         }
       }
+      flush_all();   // after at most 32 members
     }
-    __syncthreads();
-    cnt = s_n;
-    rows(cnt, [&](int m) { return (int64_t)s_list[m]; });
+  };
+  const uint8_t* asg = a.asg + (size_t)h * a.N;
+  if (cnt <= a.cap) {
+    const size_t at = (size_t)w * a.cap;
+    if (a.wide) rows(cnt, [&](int i) { return (int64_t)reinterpret_cast<const int32_t*>(a.list)[at + i]; });
+    else rows(cnt, [&](int i) { return (int64_t)reinterpret_cast<const uint16_t*>(a.list)[at + i]; });
   } else {
-    cnt = a.counts[w];
-    const int base = a.offs[w];
-    const int32_t* lst = a.list + (size_t)h * a.N + (base < a.N ? base : 0);
-    rows(cnt, [&](int m) { return (int64_t)lst[m]; });
+    const uint32_t jj = (uint32_t)j * 0x01010101u;
+    const int lead = (int)(reinterpret_cast<uintptr_t>(asg) & 15u);   // the head's bytes start inside a 16-byte word
+    for (int64_t c0 = 0; c0 < a.N; c0 += kPick) {
+      const int64_t c1 = c0 + kPick < a.N ? c0 + kPick : a.N;
+      // whole words over tokens [c0, c1) (kPick is a multiple of 16)
+      for (int64_t o = c0 - lead + 16 * tid; o < c1; o += 16 * 128) {
+        const uint4 v = *reinterpret_cast<const uint4*>(asg + o);
+        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t mk = __vcmpeq4(w4[q], jj) & 0x01010101u;
+          while (mk) {
+            const int64_t t = o + 4 * q + ((__ffs((int)mk) - 1) >> 3);
+            mk &= mk - 1;
+            if (t >= c0 && t < c1) s_list[atomicAdd(&s_n, 1)] = (uint16_t)(t - c0);
+          }
+        }
+      }
+      __syncthreads();
+      const int n = s_n;
+      rows(n, [&](int i) { return c0 + (int64_t)s_list[i]; });
+      __syncthreads();
+      if (tid == 0) s_n = 0;
+      __syncthreads();
+    }
   }
-  flush(k0, 0);
-  flush(k1, 1);
-  flush(k2, 2);
-  flush(k3, 3);
   s_sum[warp][4 * lane] = k0;
   s_sum[warp][4 * lane + 1] = k1;
   s_sum[warp][4 * lane + 2] = k2;
   s_sum[warp][4 * lane + 3] = k3;
-  if (!grid_ok) s_ok = 0;
+  {
+    const uint32_t lim = ((uint32_t)(U + 134) << 7) - 1u;   // magnitude - 1 of the smallest value on the grid
+    const bool on_grid = most == 0u || (U >= -127 && min(least & 0xFFFFu, least >> 16) >= lim &&
+                                        max(most & 0xFFFFu, most >> 16) < 0x7F80u);
+    if (!on_grid) s_ok = 0;
+  }
   __syncthreads();
   if (warp != 0) return;
 
-  float4* cr = reinterpret_cast<float4*>(a.cent + (size_t)w * 128) + lane;
-  float4 m = *cr;
   if (cnt > 0) {
     const double dc = (double)cnt;
     bool ok = s_ok != 0 && cnt <= (1 << 24);
@@ -673,26 +663,17 @@ __global__ void __launch_bounds__(128) fit_means(const FitArgs a, int last) {
         m = make_float4(mean_of(total(0), U, rh, rl, dc), mean_of(total(1), U, rh, rl, dc),
                         mean_of(total(2), U, rh, rl, dc), mean_of(total(3), U, rh, rl, dc));
     }
-    if (!ok) {  // fp64 sums (exact for members of ordinary range)
+    if (!ok) {  // fp64 sums in token order (exact for members of ordinary range)
       double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      auto add = [&](int64_t tok) {
-        const uint2 xv = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
-        s0 += (double)__uint_as_float(xv.x << 16);
-        s1 += (double)__uint_as_float(xv.x & 0xFFFF0000u);
-        s2 += (double)__uint_as_float(xv.y << 16);
-        s3 += (double)__uint_as_float(xv.y & 0xFFFF0000u);
-      };
-      if (a.scan) {
-        for (int64_t n0 = 0; n0 < a.N; n0 += 32) {
-          uint32_t mk = __ballot_sync(0xFFFFFFFFu, n0 + lane < a.N && asg[n0 + lane] == (uint8_t)j);
-          for (; mk; mk &= mk - 1) add(n0 + __ffs((int)mk) - 1);
-        }
-      } else {
-        const int base = a.offs[w];
-        const int32_t* lst = a.list + (size_t)h * a.N + (base < a.N ? base : 0);
-        for (int i = 0; i < cnt; ++i) {
-          const int64_t tok = lst[i];
-          if (tok >= 0 && tok < a.N) add(tok);
+      for (int64_t n0 = 0; n0 < a.N; n0 += 32) {
+        uint32_t mk = __ballot_sync(0xFFFFFFFFu, n0 + lane < a.N && asg[n0 + lane] == (uint8_t)j);
+        for (; mk; mk &= mk - 1) {
+          const int64_t tok = n0 + __ffs((int)mk) - 1;
+          const uint2 xv = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)tok * a.H + h) * 128 + 4 * lane));
+          s0 += (double)__uint_as_float(xv.x << 16);
+          s1 += (double)__uint_as_float(xv.x & 0xFFFF0000u);
+          s2 += (double)__uint_as_float(xv.y << 16);
+          s3 += (double)__uint_as_float(xv.y & 0xFFFF0000u);
         }
       }
       m = make_float4(__double2float_rn(__ddiv_rn(s0, dc)), __double2float_rn(__ddiv_rn(s1, dc)),
@@ -709,7 +690,7 @@ __global__ void __launch_bounds__(128) fit_means(const FitArgs a, int last) {
     return;
   }
   emit_row(a, h, j, m, lane);
-  if (lane == 0 && !a.scan) a.counts[w] = 0;  // ready for the next assignment
+  if (lane == 0) a.counts[w] = 0;  // ready for the next assignment
 }
 
 // bf16 output of the initial centroids (no iteration).
@@ -765,17 +746,13 @@ void fit_carve(FitArgs& a, uint8_t* ws) {
   while (((int64_t)1 << lg) < a.N + 1) ++lg;
   a.room = 53 - lg < 40 ? 53 - lg : 40;  // values below 2^48 units: three fp32 limbs (fit_means)
   a.counts = reinterpret_cast<int32_t*>(take((int64_t)a.H * a.C * 4));
-  a.offs = reinterpret_cast<int32_t*>(take((int64_t)a.H * a.C * 4));
+  take((int64_t)a.H * a.C * 4);   // reserved
   a.asg = take((int64_t)a.H * a.N);
   a.xn2 = reinterpret_cast<float*>(take((int64_t)a.H * a.N * 4));
   a.list = reinterpret_cast<int32_t*>(take((int64_t)a.H * a.N * 4));
-  // Up to kScanTokens tokens the means pick their members out of the assignment
-  // bytes (every centroid of a head reads them all: at 8192 tokens as much as
-  // the rows of the members), which then lie in the list's place, each head's
-  // padded to 16 bytes; beyond that the sorted list is built.
-  a.scan = a.N >= 16 && a.N <= kScanTokens;
-  a.asg_stride = a.scan ? round_up(a.N, 16) : a.N;
-  if (a.scan) a.asg = reinterpret_cast<uint8_t*>(a.list);
+  // members listed per centroid: twice the average where a token's index fits 16 bits
+  a.wide = a.N > 65536;
+  a.cap = (int32_t)((a.wide ? a.N : 2 * a.N) / a.C);
 }
 
 namespace {
@@ -817,7 +794,6 @@ cudaError_t launch_fit(const FitArgs& a, cudaStream_t st) {
   e = launch_pdl(fit_scale, dim3((unsigned)(sb < 64 ? sb : 64), (unsigned)a.H), 256, 0, st, a);
   for (int it = 0; it < a.iters && e == cudaSuccess; ++it) {
     e = launch_pdl(fit_assign, dim3((unsigned)grid), ANT, A_SMEM, st, a, tm, tiles, units);
-    if (e == cudaSuccess && !a.scan) e = launch_pdl(fit_scatter, dim3((unsigned)a.H), 1024, 0, st, a);
     if (e == cudaSuccess)
       e = launch_pdl(fit_means, dim3((unsigned)((int64_t)a.H * a.C)), 128, 0, st, a, (int)(it + 1 == a.iters));
   }

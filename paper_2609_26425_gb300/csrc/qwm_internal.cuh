@@ -221,11 +221,10 @@ struct FitArgs {
   float* xn2;                  // [H][N] |x|^2 of every token (fp32, any order)
   int room;                    // fixed-point headroom bits of the exact member sums
   int32_t* counts;             // [H][C] members per cluster
-  int32_t* offs;               // [H][C] first member slot
-  bool scan;                   // the means scan the assignment instead of reading the sorted list
-  int64_t asg_stride;
-  uint8_t* asg;                // [H][asg_stride] assignment
-  int32_t* list;               // [H][N] member token indices grouped by cluster
+  int32_t cap;                 // members listed per centroid, at most
+  bool wide;                   // list entries of 32 bits (16 otherwise)
+  uint8_t* asg;                // [H][N] assignment
+  int32_t* list;               // [H][C][cap] token indices of each centroid's members
 };
 struct DequantArgs {
   Layout L;
