@@ -47,16 +47,17 @@ using namespace ptx;
 constexpr int AT = 128;                       // tokens per tile
 constexpr int AEW = 16;                       // epilogue warps: rows 32 (w & 3) + lane, column quarter w >> 2
 constexpr int ANT = (AEW + 1) * 32;           // + one producer / MMA warp
-constexpr int kPairCap = 1024;                // (row, centroid) pairs rescored per tile
+constexpr int kPairCap = 2048;                // (token, centroid) pairs waiting to be rescored
+constexpr int kRowCapList = kPairCap / 2;     // tokens they belong to (two or more candidates each)
 constexpr int kRowCap = 8;                    // candidates per row
 constexpr int A_X = 0;                        // 2 token tiles, each 2 x [128 rows][128 B] bf16
 constexpr int A_IMG = 65536;                  // operand images hi, lo: 2 x 2 x [Npad][128 B]
 constexpr int A_ONE = A_IMG + 131072;         // ones: [128 rows][16] bf16 operand (columns 0 and 1), no swizzle
 constexpr int A_NRM = A_ONE + 4096;           // -|mu_j|^2 / 2 in two bf16 parts: [256 rows][16], no swizzle
-constexpr int A_PJ = A_NRM + 8192;            // pair (row << 16 | j) [kPairCap]
-constexpr int A_PD = A_PJ + kPairCap * 4;     // pair distance [kPairCap]
-constexpr int A_ROW = A_PD + kPairCap * 4;    // row: first slot << 16 | count (0xFFFF: full scan)
-constexpr int A_MIN = A_ROW + AT * 4;         // [4 quarters][128] partial maxima of s
+constexpr int A_PJ = A_NRM + 8192;            // waiting pairs' centroids (u8) [kPairCap]
+constexpr int A_ROW = A_PJ + kPairCap;        // waiting tokens: tile of the run << 7 | row [kRowCapList]
+constexpr int A_RPJ = A_ROW + kRowCapList * 4;   // their first pair << 4 | number of pairs [kRowCapList] (u16)
+constexpr int A_MIN = A_RPJ + kRowCapList * 2;         // [4 quarters][128] partial maxima of s
 constexpr int A_CNT = A_MIN + 4 * AT * 4;     // [4 quarters][128] candidate count | first candidate << 8
 constexpr int A_CND = A_CNT + 4 * AT * 4;     // [128][4 quarters][kRowCap] candidates (u8)
 constexpr int A_BAR = A_CND + AT * 4 * kRowCap;   // mbarriers, pair counter, flag, TMEM slot
@@ -92,21 +93,14 @@ __device__ __forceinline__ int sw_off(int rows, int row, int ch) {
 
 // The sequential fp32 distance of the definition: channel order, the
 // difference, its square and the running sum each rounded on its own.
-__device__ float exact_dist(const uint8_t* sX, int row, const float* mu) {
-  const float4* m4 = reinterpret_cast<const float4*>(mu);
-  float4 mv[16];   // a ring of 64 channels: the loads run ahead of the chain
-#pragma unroll
-  for (int i = 0; i < 16; ++i) mv[i] = __ldg(m4 + i);
+// (One thread: for rows left to the search of every centroid.)
+__device__ __noinline__ float exact_dist(const __nv_bfloat16* x, const float* mu) {
   float acc = 0.0f;
-#pragma unroll
+#pragma unroll 1
   for (int ch = 0; ch < 16; ++ch) {
-    const uint4 xv = *reinterpret_cast<const uint4*>(sX + sw_off(128, row, ch));
-    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
-    const float4 ma = mv[(2 * ch) & 15], mb = mv[(2 * ch + 1) & 15];
-    if (ch < 8) {
-      mv[2 * ch] = __ldg(m4 + 2 * ch + 16);
-      mv[2 * ch + 1] = __ldg(m4 + 2 * ch + 17);
-    }
+    const float4 ma = __ldg(reinterpret_cast<const float4*>(mu) + 2 * ch), mb = __ldg(reinterpret_cast<const float4*>(mu) + 2 * ch + 1);
+    const uint4 xr = __ldg(reinterpret_cast<const uint4*>(x) + ch);
+    const uint32_t xw[4] = {xr.x, xr.y, xr.z, xr.w};
     const float ms[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -116,6 +110,41 @@ __device__ float exact_dist(const uint8_t* sX, int row, const float* mu) {
     }
   }
   return acc;
+}
+
+// The same sum for two centroids by a warp: lane l squares channels 4 l .. 4 l
+// + 3 (the rows fetched at once), then the running sums pass through the lanes
+// in order.  Every lane gets the results.  (Its own function: inlined, its
+// registers spilled under those of the kernel's tile loop.)
+__device__ __noinline__ float2 exact_dist2(uint2 xv, const float* mu0, const float* mu1) {
+  const int lane = threadIdx.x & 31;
+  const float xf[4] = {__uint_as_float(xv.x << 16), __uint_as_float(xv.x & 0xFFFF0000u), __uint_as_float(xv.y << 16),
+                       __uint_as_float(xv.y & 0xFFFF0000u)};
+  const float4 ma = __ldg(reinterpret_cast<const float4*>(mu0) + lane), mb = __ldg(reinterpret_cast<const float4*>(mu1) + lane);
+  const float m0[4] = {ma.x, ma.y, ma.z, ma.w}, m1[4] = {mb.x, mb.y, mb.z, mb.w};
+  float s0[4], s1[4], d0 = 0.0f, d1 = 0.0f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float t0 = __fsub_rn(xf[e], m0[e]), t1 = __fsub_rn(xf[e], m1[e]);
+    s0[e] = __fmul_rn(t0, t0);
+    s1[e] = __fmul_rn(t1, t1);
+  }
+  // step l leaves lane l with the sum over the channels up to its own (the lanes
+  // after it with values that later steps replace)
+#pragma unroll 4
+  for (int l = 0; l < 32; ++l) {
+    float a = __shfl_up_sync(0xFFFFFFFFu, d0, 1), b = __shfl_up_sync(0xFFFFFFFFu, d1, 1);
+    a = lane == 0 ? 0.0f : a;
+    b = lane == 0 ? 0.0f : b;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      a = __fadd_rn(a, s0[e]);
+      b = __fadd_rn(b, s1[e]);
+    }
+    d0 = a;
+    d1 = b;
+  }
+  return make_float2(__shfl_sync(0xFFFFFFFFu, d0, 31), __shfl_sync(0xFFFFFFFFu, d1, 31));
 }
 
 // Operand images and norm of centroid j of head h from its fp32 row (one
@@ -176,16 +205,19 @@ __global__ void __launch_bounds__(512) fit_prep(const FitArgs a) {
 // (TMA) and multiplies (tcgen05) tile t + 1 into the second token buffer and
 // TMEM accumulator while warps 0-15 finish tile t: four warps per row, one per
 // column quarter of the accumulator (at most 64 columns, read once and kept in
-// registers), meeting in shared memory.
+// registers), meeting in shared memory.  The rows that need the exact distance
+// wait in a list until the run's end (or until it may not hold another tile's):
+// rescored tile by tile, a handful of rows each, their latency was a third of
+// the kernel's time.
 __global__ void __launch_bounds__(ANT, 1)
     fit_assign(const FitArgs a, const __grid_constant__ CUtensorMap tm, int tiles, int units) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int C = a.C, Npad = a.Npad;
-  uint32_t* sPJ = reinterpret_cast<uint32_t*>(sm + A_PJ);
-  float* sPD = reinterpret_cast<float*>(sm + A_PD);
+  uint8_t* sPJ = sm + A_PJ;
   uint32_t* sRow = reinterpret_cast<uint32_t*>(sm + A_ROW);
+  uint16_t* sRpj = reinterpret_cast<uint16_t*>(sm + A_RPJ);
   float* sMin = reinterpret_cast<float*>(sm + A_MIN);
   int* sCnt = reinterpret_cast<int*>(sm + A_CNT);
   uint8_t* sCnd = sm + A_CND;
@@ -194,7 +226,7 @@ __global__ void __launch_bounds__(ANT, 1)
   auto bar_mma = [&](int b) { return bars + 16 + 8 * b; };     // accumulator b complete
   auto bar_free = [&](int b) { return bars + 32 + 8 * b; };    // tile b and accumulator b consumed
   const uint32_t bar_img = bars + 48;
-  int* s_np = reinterpret_cast<int*>(sm + A_BAR + 64);
+  int* s_np = reinterpret_cast<int*>(sm + A_BAR + 64);   // pairs waiting; s_np[3]: tokens waiting
   volatile int* s_err = reinterpret_cast<volatile int*>(sm + A_BAR + 68);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + A_BAR + 72);
   uint32_t ncols = 32;
@@ -223,7 +255,7 @@ __global__ void __launch_bounds__(ANT, 1)
     }
     mbar_init(bar_img, 1);
     fence_mbar_init();
-    *s_np = 0;
+    s_np[0] = s_np[3] = 0;
     *s_err = 0;
   }
   tc_fence_before();
@@ -243,20 +275,21 @@ __global__ void __launch_bounds__(ANT, 1)
     int cur_h = -1;
     uint32_t ph_img = 0;
     bool go = true;
-    for (int t = 0; t < T && go; ++t) {
-      const int u = u0 + t, h = u / tiles, tile = u - h * tiles, b = t & 1;
-      if (t >= 2) go = __all_sync(0xFFFFFFFFu, mbar_wait(bar_free(b), ((t >> 1) - 1) & 1));
-      const bool copying = go;
+    auto load_tile = [&](int t) {
+      const int u = u0 + t, h = u / tiles, b = t & 1;
       const uint32_t aX = smem_u32(sm + A_X + b * 32768);
-      if (go && lane == 0) {
+      if (lane == 0) {
         mbar_arrive_expect_tx(bar_tma(b), 32768u);
-        tma_load_3d(aX, &tm, 0, h, tile * 128, bar_tma(b));
-        tma_load_3d(aX + 16384, &tm, 64, h, tile * 128, bar_tma(b));
+        tma_load_3d(aX, &tm, 0, h, (u - h * tiles) * 128, bar_tma(b));
+        tma_load_3d(aX + 16384, &tm, 64, h, (u - h * tiles) * 128, bar_tma(b));
       }
-      if (go && h != cur_h) {
+    };
+    if (T > 0) load_tile(0);
+    for (int t = 0; t < T; ++t) {
+      const int h = (u0 + t) / tiles, b = t & 1;
+      if (h != cur_h) {
         // the previous head's MMAs read the images and norms: wait for them, then load this head's
-        if (t >= 1) go = mbar_wait(bar_mma((t - 1) & 1), ((t - 1) >> 1) & 1);
-        go = __all_sync(0xFFFFFFFFu, go);
+        if (t >= 1) go = __all_sync(0xFFFFFFFFu, mbar_wait(bar_mma((t - 1) & 1), ((t - 1) >> 1) & 1));
         if (go) {
           if (lane == 0) {
             mbar_arrive_expect_tx(bar_img, (uint32_t)Npad * 512u);
@@ -272,15 +305,17 @@ __global__ void __launch_bounds__(ANT, 1)
           cur_h = h;
         }
       }
-      if (go) go = mbar_wait(bar_tma(b), (t >> 1) & 1);
+      go = go && mbar_wait(bar_tma(b), (t >> 1) & 1);
+      go = go && (t < 2 || mbar_wait(bar_free(b), ((t >> 1) - 1) & 1));
       go = __all_sync(0xFFFFFFFFu, go);
       if (!go) {
-        if (copying) mbar_wait(bar_tma(b), (t >> 1) & 1);   // no copy outlives the CTA
+        mbar_wait(bar_tma(b), (t >> 1) & 1);   // no copy outlives the CTA
         *s_err = 1;
         break;
       }
       tc_fence_after();
       if (lane == 0) {
+        const uint32_t aX = smem_u32(sm + A_X + b * 32768);
         const uint32_t tD = tbase + (uint32_t)b * ncols;
 #pragma unroll
         for (int half = 0; half < 2; ++half)
@@ -294,6 +329,15 @@ __global__ void __launch_bounds__(ANT, 1)
         umma_commit(bar_mma(b));
       }
       __syncwarp();
+      // the next tile's copy, once the MMAs of the tile before this one have left its buffer
+      if (t + 1 < T) {
+        if (t >= 1) go = __all_sync(0xFFFFFFFFu, mbar_wait(bar_mma(b ^ 1), ((t - 1) >> 1) & 1));
+        if (!go) {
+          *s_err = 1;
+          break;
+        }
+        load_tile(t + 1);
+      }
     }
   } else {
     // ---------------- epilogue: warps 0-15
@@ -301,8 +345,8 @@ __global__ void __launch_bounds__(ANT, 1)
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
     const int nchunk = (Npad + 31) >> 5;
     const int ch0 = (qt * nchunk) >> 2, ch1 = ((qt + 1) * nchunk) >> 2;   // this quarter's 32-column chunks
-    // A token's place among its centroid's members comes back from an atomic
-    // count; it is listed one tile later, when that has long arrived.
+    // A token's assignment.  Its place among its centroid's members comes back
+    // from an atomic count; it is listed one call later, when that has long arrived.
     int pl_rank = 0, pl_tok = -1;
     size_t pl_cent = 0;
     auto list_member = [&]() {
@@ -311,17 +355,50 @@ __global__ void __launch_bounds__(ANT, 1)
       if (a.wide) reinterpret_cast<int32_t*>(a.list)[at] = pl_tok;
       else reinterpret_cast<uint16_t*>(a.list)[at] = (uint16_t)pl_tok;
     };
+    auto assign = [&](int h, int64_t n, int j) {
+      a.asg[(size_t)h * a.N + n] = (uint8_t)j;
+      list_member();
+      pl_cent = (size_t)h * C + j;
+      pl_tok = (int)n;
+      pl_rank = atomicAdd(a.counts + pl_cent, 1);
+    };
+    // the waiting tokens' exact distances, a warp each: ascending centroids, the
+    // lower one keeps a tie (called by all epilogue threads, the list complete)
+    auto rescore = [&]() {
+      const int nr = s_np[3];
+#pragma unroll 1
+      for (int r = warp; r < nr; r += AEW) {
+        const int u = u0 + (int)(sRow[r] >> 7), h = u / tiles;
+        const int64_t n = (int64_t)(u - h * tiles) * 128 + (sRow[r] & 127u);
+        const int p0 = sRpj[r] >> 4, np = sRpj[r] & 15;
+        const uint2 xv = __ldg(reinterpret_cast<const uint2*>(a.x + ((size_t)n * a.H + h) * 128) + lane);
+        float bd = 0.0f;
+        int best = -1;
+#pragma unroll 1
+        for (int p = 0; p < np; p += 2) {
+          const int j0 = sPJ[p0 + p], j1 = sPJ[p0 + min(p + 1, np - 1)];
+          const float* cent = a.cent + (size_t)h * C * 128;
+          const float2 d = exact_dist2(xv, cent + j0 * 128, cent + j1 * 128);
+          if (best < 0 || d.x < bd) {
+            bd = d.x;
+            best = j0;
+          }
+          if (d.y < bd) {
+            bd = d.y;
+            best = j1;
+          }
+        }
+        if (lane == 0) assign(h, n, best);
+      }
+    };
     for (int t = 0; t < T; ++t) {
       const int u = u0 + t, h = u / tiles, tile = u - h * tiles, b = t & 1;
-      const uint8_t* sX = sm + A_X + b * 32768;
       const uint32_t tD = tbase + (uint32_t)b * ncols;
       const int64_t n = (int64_t)tile * 128 + row;
       const bool valid = n < a.N;
       const float kx = valid ? a.xn2[(size_t)h * a.N + n] : 0.0f;
-      bool ok = mbar_wait(bar_mma(b), (t >> 1) & 1);
-      ok = __all_sync(0xFFFFFFFFu, ok);
+      const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar_mma(b), (t >> 1) & 1));
       tc_fence_after();
-      if (!ok) *s_err = 1;
       // s_j of this quarter's columns and the largest
       constexpr float kC = 1.220703125e-4f;   // c
       float v[64];
@@ -333,7 +410,13 @@ __global__ void __launch_bounds__(ANT, 1)
       }
       sMin[qt * AT + row] = mx;
       tc_fence_before();
-      named_bar_sync(1, AEW * 32);
+      if (lane == 0) mbar_arrive(bar_free(b));   // the accumulator is in registers
+      // one vote, so that every epilogue warp leaves the loop together
+      if (!named_bar_and(1, AEW * 32, ok)) {
+        *s_err = 1;
+        break;
+      }
+      const bool full = s_np[0] > kPairCap - AT * kRowCap;   // the list may not hold this tile's pairs
       mx = fmaxf(fmaxf(sMin[row], sMin[AT + row]), fmaxf(sMin[2 * AT + row], sMin[3 * AT + row]));
       const float dist = fmaxf(fmaf(-2.0f, mx, kx), 0.0f);
       const float thr = fmaf(-kC, fmaf(2.02f, kx + dist, kx), mx) - 1e-30f;
@@ -365,11 +448,16 @@ __global__ void __launch_bounds__(ANT, 1)
       }
       sCnt[qt * AT + row] = (int)word;
       named_bar_sync(1, AEW * 32);
-      // the row owner (quarter 0) merges: one candidate decides, a few go to the pair list
-      int best = 0;
-      if (qt == 0) {
+      if (full) {
+        rescore();
+        named_bar_sync(1, AEW * 32);
+        if (tid == 0) s_np[0] = s_np[3] = 0;
+        named_bar_sync(1, AEW * 32);
+      }
+      // the row owner (quarter 0) merges: one candidate decides, a few wait for their exact distances
+      if (qt == 0 && valid) {
         uint32_t cw[4];
-        int tot = 0;
+        int tot = 0, best = 0;
         bool bad = false;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -378,72 +466,39 @@ __global__ void __launch_bounds__(ANT, 1)
           tot += (int)(cw[q] & 0xFFu);
           if (cw[q] & 0xFFu) best = (int)(cw[q] >> 8);
         }
-        uint32_t rinfo = 0;
-        if (bad || tot == 0 || tot > kRowCap) {
-          rinfo = 0xFFFFu;  // every centroid, sequentially
-        } else if (tot > 1 && valid) {
-          const int base = atomicAdd(s_np, tot);
-          if (base + tot <= kPairCap) {
-            int s2 = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int n2 = (int)(cw[q] & 0xFFu);
-              for (int k = 0; k < n2; ++k)
-                sPJ[base + s2++] =
-                    ((uint32_t)row << 16) | (n2 == 1 ? cw[q] >> 8 : (uint32_t)sCnd[(row * 4 + q) * kRowCap + k]);
-            }
-            rinfo = ((uint32_t)base << 16) | (uint32_t)tot;
-          } else {
-            rinfo = 0xFFFFu;
-          }
-        }
-        sRow[row] = rinfo;
-      }
-      named_bar_sync(1, AEW * 32);
-      // exact rescoring of the listed pairs, spread over the epilogue warps
-      const int np = min(*s_np, kPairCap);
-      const float* muh = a.cent + (size_t)h * C * 128;
-      for (int p = tid; p < np; p += AEW * 32) {
-        const uint32_t pj = sPJ[p];
-        sPD[p] = exact_dist(sX, (int)(pj >> 16), muh + (size_t)(pj & 0xFFFFu) * 128);
-      }
-      if (np > 0) named_bar_sync(1, AEW * 32);   // np is the same for every thread
-      if (qt == 0 && valid && ok) {
-        const uint32_t rinfo = sRow[row];
-        if (rinfo == 0xFFFFu) {
+        if (bad || tot == 0 || tot > kRowCap) {   // every centroid, sequentially
+          const __nv_bfloat16* xr = a.x + ((size_t)n * a.H + h) * 128;
           float bd = 0.0f;
           for (int j = 0; j < C; ++j) {
-            const float dj = exact_dist(sX, row, muh + (size_t)j * 128);
+            const float dj = exact_dist(xr, a.cent + ((size_t)h * C + j) * 128);
             if (j == 0 || dj < bd) {
               bd = dj;
               best = j;
             }
           }
-        } else if (rinfo != 0) {
-          const int base = (int)(rinfo >> 16), c2 = (int)(rinfo & 0xFFFFu);
-          float bd = sPD[base];
-          best = (int)(sPJ[base] & 0xFFFFu);
-          for (int s2 = 1; s2 < c2; ++s2)
-            if (sPD[base + s2] < bd) {  // ascending j: the lower index keeps a tie
-              bd = sPD[base + s2];
-              best = (int)(sPJ[base + s2] & 0xFFFFu);
-            }
+          tot = 1;
         }
-        a.asg[(size_t)h * a.N + n] = (uint8_t)best;
-        list_member();
-        pl_cent = (size_t)h * C + best;
-        pl_tok = (int)n;
-        pl_rank = atomicAdd(a.counts + pl_cent, 1);
+        if (tot == 1) {
+          assign(h, n, best);
+        } else {
+          const int p0 = atomicAdd(s_np, tot), r = atomicAdd(s_np + 3, 1);
+          int k = p0;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int n2 = (int)(cw[q] & 0xFFu);
+            for (int c2 = 0; c2 < n2; ++c2)
+              sPJ[k++] = n2 == 1 ? (uint8_t)(cw[q] >> 8) : sCnd[(row * 4 + q) * kRowCap + c2];
+          }
+          sRow[r] = ((uint32_t)t << 7) | (uint32_t)row;
+          sRpj[r] = (uint16_t)((p0 << 4) | tot);
+        }
       }
-      fence_proxy_async_smem();  // generic reads of tile b before the next copy into it
-      tc_fence_before();
-      // one vote, so that every epilogue warp leaves the loop together
-      const bool go = named_bar_and(1, AEW * 32, *s_err == 0);
-      if (tid == 0) *s_np = 0;
-      if (lane == 0) mbar_arrive(bar_free(b));
-      if (!go) break;
+      if (t == T - 1) {
+        named_bar_sync(1, AEW * 32);
+        rescore();
+      }
     }
-    if (qt == 0) list_member();
+    list_member();
   }
   if (tid == 0 && *s_err) atomicCAS(a.status, 0, (int)QWM_ERR_TIMEOUT);
   tc_fence_before();
