@@ -36,6 +36,8 @@
 // The selection of the full quadratic form (App. C.4) and the exhaustive
 // range 8 < M < C use the other append kernels.
 #pragma once
+#include <type_traits>
+
 #include "ptx_sm103.cuh"
 #include "qwm_internal.cuh"
 #include "append_common.cuh"
@@ -102,13 +104,67 @@ __device__ __forceinline__ float dq_smem(const uint8_t* rows, int r, const uint8
   return acc;
 }
 
+// The units of each CTA: [first[b], first[b + 1]).
+constexpr int kMaxCtas = 256;
+struct FusedShares {
+  int32_t first[kMaxCtas + 1];
+};
+
+// Shares of `units` (2 * pairs runs of `tiles`, Keys first) over at most `ctas`
+// CTAs with the smallest longest time (Wan-14B chunk 367 -> 328 us, 16001 tokens
+// at r = 32, M = 8: 3.19 -> 2.67 ms, against equal shares): a CTA's runs come one after another, each
+// taking kSetup and the tiles of the group that has more of them.  A Key tile
+// costs more than a Value tile, and with equal shares the CTAs on Values idled
+// for the difference.  The time is found by trials, each CTA in turn taking
+// what fits in it (host arithmetic, about 250 steps a trial, fewer than ten).
+inline int fused_shares(FusedShares& sh, int units, int tiles, int ctas, int kcost, int vcost) {
+  constexpr int64_t kSetup = 5;
+  const int nkey = units / 2;
+  auto fill = [&](int64_t limit) -> int {   // CTAs used, or ctas + 1
+    int u = 0, b = 0;
+    while (u < units) {
+      if (b == ctas) return ctas + 1;
+      sh.first[b++] = u;
+      for (int64_t used = 0; u < units;) {
+        const int64_t c = u < nkey ? kcost : vcost;
+        const int64_t slots = (limit - used - kSetup) / c;
+        if (slots <= 0) break;
+        const int rest = tiles - u % tiles, take = rest < 2 * slots ? rest : (int)(2 * slots);
+        used += kSetup + (take + 1) / 2 * c;
+        u += take;
+        if (take < rest) break;
+      }
+    }
+    for (int e = b; e <= ctas; ++e) sh.first[e] = units;
+    return b;
+  };
+  // one unit per CTA always fits in a Key tile's time when the CTAs suffice
+  if (units <= ctas) {
+    for (int b = 0; b <= ctas; ++b) sh.first[b] = b < units ? b : units;
+    return units;
+  }
+  // from the mean share of a group upwards, to within 1 %
+  const int64_t most = kSetup + (kcost > vcost ? kcost : vcost), mean = (int64_t)nkey * (kcost + vcost) / (2 * ctas);
+  int64_t lo = mean > most ? mean : most, hi = lo;
+  while (fill(hi) > ctas) {
+    lo = hi + 1;
+    hi += hi / 16 + 1;
+  }
+  while (hi - lo > hi / 128) {
+    const int64_t mid = (lo + hi) / 2;
+    if (fill(mid) <= ctas) hi = mid;
+    else lo = mid + 1;
+  }
+  return fill(hi);
+}
+
 // CAPT = M + 1 (the ranked list of a row; kMaxFilterM + 1 for the candidate
 // counts without their own instance), R = PSAC rank.
 template <int CAPT, int R>
 __global__ void __launch_bounds__(XNT, 1)
     append_fused(const AppendArgs a, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kc,
-                 const __grid_constant__ CUtensorMap tm_vc, int tiles, int units) {
+                 const __grid_constant__ CUtensorMap tm_vc, const __grid_constant__ FusedShares shares, int tiles) {
   using S = XSmem<R>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -159,11 +215,9 @@ __global__ void __launch_bounds__(XNT, 1)
   const uint32_t tD = tbase + (uint32_t)(g * 256);
   const uint32_t lrow = (uint32_t)(gw * 32) << 16;
 
-  // Work unit u = (side * H + h) * tiles + tile; this CTA takes [u0, u1), a
-  // run per (head, side); group g takes the units u0 + g, u0 + g + 2, ...
-  const int nb = gridDim.x;
-  const int u0 = (int)((int64_t)blockIdx.x * units / nb);
-  const int u1 = (int)((int64_t)(blockIdx.x + 1) * units / nb);
+  // Work unit u = (side * H + h) * tiles + tile, Keys first; this CTA takes
+  // [u0, u1), a run per (head, side); group g takes the units u0 + g, u0 + g + 2, ...
+  const int u0 = shares.first[blockIdx.x], u1 = shares.first[blockIdx.x + 1];
   auto issue_tile = [&](int u) {
     const int pr = u / tiles, tl = u - pr * tiles;
     const CUtensorMap* tm = pr < H ? &tm_k : &tm_v;
@@ -690,8 +744,11 @@ __global__ void __launch_bounds__(XNT, 1)
 #pragma unroll
         for (int gi = 0; gi < 4; ++gi) { bmn[gi] = 0.0f; bmx[gi] = 0.0f; }
         const int ncand = all_cand ? C : Mc;
-        for (int m0 = 0; m0 < ncand; m0 += QB) {
-          const int nbq = ncand - m0 < QB ? ncand - m0 : QB;
+        // a whole batch of QB candidates has no branch per candidate, so that
+        // the loads of one run under the arithmetic of another
+        auto score = [&](auto whole, int m0) {
+          constexpr bool kWhole = decltype(whole)::value;
+          const int nbq = kWhole ? QB : ncand - m0;
           int jb[QB];
 #pragma unroll
           for (int b = 0; b < QB; ++b) {
@@ -714,7 +771,6 @@ __global__ void __launch_bounds__(XNT, 1)
           for (int cc = 0; cc < 8; ++cc) {
             const int qq = cc >> 1;
             uint64_t k2[8];
-#pragma unroll
             {
               const uint4 ka = row_chunk(myrow, rkey, 2 * cc), kb = row_chunk(myrow, rkey, 2 * cc + 1);
               const uint32_t kw[8] = {ka.x, ka.y, ka.z, ka.w, kb.x, kb.y, kb.z, kb.w};
@@ -723,7 +779,7 @@ __global__ void __launch_bounds__(XNT, 1)
             }
 #pragma unroll
             for (int b = 0; b < QB; ++b) {
-              if (b < nbq) {
+              if (kWhole || b < nbq) {
                 const uint4 ma = lds16(sMU + sw_off(Npad, jb[b], 2 * cc));
                 const uint4 mb = lds16(sMU + sw_off(Npad, jb[b], 2 * cc + 1));
                 const uint32_t mw[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
@@ -740,7 +796,7 @@ __global__ void __launch_bounds__(XNT, 1)
           }
 #pragma unroll
           for (int b = 0; b < QB; ++b) {
-            if (b < nbq) {
+            if (kWhole || b < nbq) {
               if (!gs32) {
                 mx[b][0] = fmaxf(mx[b][0], mx[b][1]);
                 mn[b][0] = fminf(mn[b][0], mn[b][1]);
@@ -764,6 +820,10 @@ __global__ void __launch_bounds__(XNT, 1)
               }
             }
           }
+        };
+        for (int m0 = 0; m0 < ncand; m0 += QB) {
+          if (ncand - m0 >= QB) score(std::true_type(), m0);
+          else score(std::false_type(), m0);
         }
         id = bestj < C ? bestj : C - 1;
 
@@ -1125,8 +1185,15 @@ cudaError_t launch_fused_rank(const AppendArgs& a, const CUtensorMap* maps, cuda
   if (e != cudaSuccess) return e;
   const int tiles = (int)((a.N + 127) / 128);
   const int units = 2 * a.L.H * tiles;
-  const int grid = units < nsm ? units : nsm;
-  kern<<<grid, XNT, smem, st>>>(a, maps[0], maps[1], maps[2], maps[3], tiles, units);
+  // Cost of a Value and a Key tile in K cycles (clock probes at C 16 to 256, r 0
+  // to 32, M 1 to 8): the selection grows with C, more than four candidates take
+  // a second scoring round and a longer ranked list, and Keys add the weighted
+  // operand and the PSAC projection.
+  const int vcost = 40 + a.L.C / 16 + (a.M > 4 ? 40 : 0);
+  const int kcost = vcost + (a.U ? (R == 8 ? 11 : R == 16 ? 20 : 46) : a.w ? 3 : 0);
+  FusedShares sh;
+  const int grid = fused_shares(sh, units, tiles, nsm < kMaxCtas ? nsm : kMaxCtas, kcost, vcost);
+  kern<<<grid, XNT, smem, st>>>(a, maps[0], maps[1], maps[2], maps[3], sh, tiles);
   return cudaGetLastError();
 }
 
