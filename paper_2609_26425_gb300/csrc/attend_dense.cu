@@ -18,14 +18,15 @@
 // read by ceil(Nq / 256) query blocks (19 at the Wan-14B layer) and inside the
 // attention kernel (attend.cu) the rebuild took issue slots and memory pipes
 // from the softmax and MMA warps in each of them.  Wan-14B layer (4680 queries,
-// 32760 keys, 40 heads), whole call: 3.67 ms there, 2.14-2.23 ms here (rebuild
-// 0.19, attention 1.87 ms = 1.67 PFLOP/s of MMA work; the longer figure under
+// 32760 keys, 40 heads), whole call: 3.67 ms there, 2.14-2.24 ms here (rebuild
+// 0.18, attention 1.87 ms = 1.67 PFLOP/s of MMA work; the longer figure under
 // the power cap of back-to-back calls); 15 x 880 + 880 keys, 880 queries, 12
-// heads: 154 -> 126 us; 4 heads, 880 queries, 2640 keys: 42 -> 31 us.
+// heads: 154 -> 109 us; 4 heads, 880 queries, 2640 keys: 42 -> 31 us; 1024
+// queries over 66544 keys, 40 heads: 1.62 -> 1.24 ms.
 //
-// The rebuild writes 512 bytes per token and head and is bound by the latency
-// of its packed reads (16 warps an SM); its bulk stores alone take 111 us at
-// the Wan-14B layer (6.0 TB/s).  The attention kernel runs at the tensor
+// The rebuild writes 512 bytes per token and head; its bulk stores alone take
+// 111 us at the Wan-14B layer (6.0 TB/s), the whole kernel 178: it waits for the
+// centroid rows (16 warps an SM).  The attention kernel runs at the tensor
 // pipe's rate (64 cycles per 128 x 128 x 16 MMA, 32 of them a tile pair) less
 // the gaps of the softmax -> MMA chain: 3.0 K cycles per 128 keys against 2.05 K.
 // One CTA per 256 queries (cta_group::1) rather than pairs: hand-offs stay
@@ -51,7 +52,6 @@ __device__ __forceinline__ void ldg32B(const void* p, uint32_t (&r)[8]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "l"(p));
 }
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // Programmatic dependent launch: let the next kernel of the stream start its
 // prologue / wait until the kernels before this one have completed.
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -110,6 +110,8 @@ constexpr int kUStride = 20;             // words per U row in shared memory (16
 // leave as bulk copies (a contiguous range of each block of the image): written
 // from registers, 16 or 32 bytes a lane, the images went out at 3.0 TB/s.
 constexpr int kStage = 8192;
+constexpr int kRecord = 15360;            // a tile's packed record, at most (15104 bytes at G = 32, r = 32)
+constexpr int kRebSmem = kRebThreads / 32 * kStage + 2 * kRecord;
 __device__ __forceinline__ void stage_row(uint8_t* stg, int i, int xr, int t, int sl, uint4 lo, uint4 hi) {
   const int sw = ((xr & 7) ^ (2 * t)) << 4;   // chunks 2 t, 2 t + 1 of image row xr
   uint8_t* d = stg + sl * 4096 + i * 128;
@@ -141,23 +143,23 @@ __device__ __forceinline__ void row_scales(const uint8_t* sp, const uint8_t* s2p
                                            uint32_t& s1) {
   if constexpr (SF == 0) {
     if (ng == 4) {
-      const uint2 x = __ldg(reinterpret_cast<const uint2*>(sp) + row);
+      const uint2 x = reinterpret_cast<const uint2*>(sp)[row];
       s0 = (t & 2) ? x.x >> 16 : x.x & 0xFFFFu;
       s1 = (t & 2) ? x.y >> 16 : x.y & 0xFFFFu;
     } else {
-      const uint32_t x = __ldg(reinterpret_cast<const uint32_t*>(sp) + row);
+      const uint32_t x = reinterpret_cast<const uint32_t*>(sp)[row];
       s0 = x & 0xFFFFu;
       s1 = x >> 16;
     }
   } else {
-    const __half s2 = __ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(s2p) + row));
+    const __half s2 = __ushort_as_half(reinterpret_cast<const unsigned short*>(s2p)[row]);
     uint32_t c0, c1;
     if (ng == 4) {
-      const uint32_t x = __ldg(reinterpret_cast<const uint32_t*>(sp) + row);
+      const uint32_t x = reinterpret_cast<const uint32_t*>(sp)[row];
       c0 = (t & 2) ? (x >> 8) & 0xFFu : x & 0xFFu;
       c1 = (t & 2) ? x >> 24 : (x >> 16) & 0xFFu;
     } else {
-      const uint32_t x = __ldg(reinterpret_cast<const unsigned short*>(sp) + row);
+      const uint32_t x = reinterpret_cast<const unsigned short*>(sp)[row];
       c0 = x & 0xFFu;
       c1 = x >> 8;
     }
@@ -168,7 +170,8 @@ __device__ __forceinline__ void row_scales(const uint8_t* sp, const uint8_t* s2p
 
 // One 128-token tile's fields of a side, and where its rows go.
 struct RebTile {
-  const uint8_t *codes, *scales, *s2, *tab, *coef, *sigma;
+  const uint8_t *codes, *scales, *s2, *coef, *sigma;   // of the record's copy in shared memory
+  const uint8_t* tab;   // centroid table (global), the lane's 32-byte slice
   uint4 pm;             // PSAC keep mask
   uint32_t idz;         // id | zero-points << 8 of this warp's row lane
   int r0, nv, ng;       // first row of the warp, rows of the tile, groups per row
@@ -202,21 +205,21 @@ __device__ __forceinline__ void rebuild_rows(const RebTile& x, const uint32_t* s
       ldg32B(mu, mv[p][0]);
       ldg32B(mu + 128, mv[p][1]);
       const uint32_t* cw = reinterpret_cast<const uint32_t*>(x.codes + rw * 32) + t;
-      word[p][0] = __ldg(cw);
-      word[p][1] = __ldg(cw + 4);
+      word[p][0] = cw[0];
+      word[p][1] = cw[4];
       row_scales<SF>(x.scales, x.s2, rw, x.ng, t, sc[p][0], sc[p][1]);
       if constexpr (RK > 0) {
         ca[0][p] = ca[0][2 + p] = ca[1][p] = ca[1][2 + p] = 0u;
         const int e = row < x.nv ? psac_entry(x.pm, row) : -1;
         if (e >= 0) {
-          const unsigned short sb = __ldg(reinterpret_cast<const unsigned short*>(x.sigma) + e);
+          const unsigned short sb = reinterpret_cast<const unsigned short*>(x.sigma)[e];
           const __half2 sg2 = u2h((uint32_t)sb | ((uint32_t)sb << 16));
           const unsigned short* cp = reinterpret_cast<const unsigned short*>(x.coef + e * RK) + t;
-          ca[0][p] = coef_f16x2(__ldg(cp), sg2);
-          if constexpr (RK > 8) ca[0][2 + p] = coef_f16x2(__ldg(cp + 4), sg2);
+          ca[0][p] = coef_f16x2(cp[0], sg2);
+          if constexpr (RK > 8) ca[0][2 + p] = coef_f16x2(cp[4], sg2);
           if constexpr (RK > 16) {
-            ca[1][p] = coef_f16x2(__ldg(cp + 8), sg2);
-            ca[1][2 + p] = coef_f16x2(__ldg(cp + 12), sg2);
+            ca[1][p] = coef_f16x2(cp[8], sg2);
+            ca[1][2 + p] = coef_f16x2(cp[12], sg2);
           }
         }
       }
@@ -280,7 +283,9 @@ __device__ __forceinline__ void rebuild_rows(const RebTile& x, const uint32_t* s
 // runs `tpc` tiles of one chunk and head.
 template <int SF, int R>
 __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs a, const AttendSlots S, int tpc) {
-  extern __shared__ __align__(16) uint8_t s_stage[];   // kStage bytes per warp
+  extern __shared__ __align__(128) uint8_t s_stage[];   // kStage bytes per warp, then two packed records
+  uint8_t* s_rec = s_stage + kRebThreads / 32 * kStage;
+  __shared__ __align__(8) uint64_t s_bar[2];            // record copied
   __shared__ uint32_t sU[R > 0 ? 128 * kUStride : 1];
   pdl_launch();
   const Layout& L = a.L;
@@ -295,6 +300,20 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
   const uint8_t* hb = cached ? a.base + head_offset(L, S.slot[u], h) : nullptr;
   const bool psac = R > 0 && cached && S.psac[u];
   bool bad = false;
+  // The packed records come by bulk copies, a tile ahead: read from global
+  // memory in the warps, their latency (twice a tile) bound the kernel.
+  auto fetch = [&](int tl) {
+    const int b = (tl - tl0) & 1;
+    mbar_arrive_expect_tx(smem_u32(s_bar + b), (uint32_t)L.tile_bytes);
+    bulk_g2s(smem_u32(s_rec + b * kRecord), hb + L.tiles_off + (int64_t)tl * L.tile_bytes, (uint32_t)L.tile_bytes,
+             smem_u32(s_bar + b));
+  };
+  if (cached && tid == 0) {
+    mbar_init(smem_u32(s_bar), 1);
+    mbar_init(smem_u32(s_bar + 1), 1);
+    fence_mbar_init();
+    fetch(tl0);
+  }
   if constexpr (R > 0) {
     if (psac) {
       // U_r^T [r][128] as binary16 into rows of MMA columns n' = 8 b + n, r values each
@@ -310,10 +329,10 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
           su[(np + 1) * (2 * kUStride) + k] = (unsigned short)(w4[e] >> 16);
         }
       }
-      __syncthreads();
     }
   }
   const int r0 = (warp & 3) * 32;        // this warp's rows of each tile
+  bool late = false;                     // a wait ran out (what follows is not used, but stays in bounds: id 0)
   for (int tl = tl0; tl < tl1; ++tl) {
     const int nv = min(128, ntok - tl * 128);
     const int64_t key0 = a.key0[u] + tl * 128;     // the tile's first key among the packed keys
@@ -346,7 +365,12 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
       store_rows(x.stg, img + (size_t)(key0 >> 7) * kImgTile, x.key0 + r0, n, lane);
       continue;
     }
-    const uint8_t* tb = hb + L.tiles_off + (int64_t)tl * L.tile_bytes;
+    uint4 pm = make_uint4(0u, 0u, 0u, 0u);
+    if (psac && key) pm = ldg16(hb + L.pmask + (int64_t)tl * 16);
+    __syncthreads();   // U_r and the barriers are in place; every warp is done with the record before
+    if (tid == 0 && tl + 1 < tl1) fetch(tl + 1);
+    if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(s_bar + ((tl - tl0) & 1)), ((tl - tl0) >> 1) & 1, a.wait_ns))) late = true;
+    const uint8_t* tb = s_rec + ((tl - tl0) & 1) * kRecord;
     x.codes = tb + (key ? L.k_codes : L.v_codes);
     x.scales = tb + (key ? L.k_scales : L.v_scales);
     x.s2 = tb + (key ? L.k_s2 : L.v_s2);
@@ -356,14 +380,12 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
     x.r0 = r0;
     x.nv = nv;
     x.ng = L.ng;
-    if (tl + 1 < tl1)   // the next tile's record towards L2
-      for (int o = tid * 64; o < (int)L.tile_bytes; o += kRebThreads * 64) prefetch_l2(tb + L.tile_bytes + o);
     x.idz = 0u;
-    if (r0 + lane < nv)
-      x.idz = (uint32_t)__ldg(tb + (key ? L.k_ids : L.v_ids) + r0 + lane) |
-              ((uint32_t)__ldg(tb + (key ? L.k_zeros : L.v_zeros) + (r0 + lane) * L.zb) << 8);
+    if (r0 + lane < nv && !late)
+      x.idz = (uint32_t)tb[(key ? L.k_ids : L.v_ids) + r0 + lane] |
+              ((uint32_t)tb[(key ? L.k_zeros : L.v_zeros) + (r0 + lane) * L.zb] << 8);
     if (psac && key) {
-      x.pm = ldg16(hb + L.pmask + (int64_t)tl * 16);
+      x.pm = pm;
       rebuild_rows<SF, R>(x, sU, lane);
     } else {
       rebuild_rows<SF, 0>(x, sU, lane);
@@ -380,6 +402,7 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
         *reinterpret_cast<uint4*>(d + (sl >> 1) * 16384 + (sl & 1) * 16) = make_uint4(0u, 0u, 0u, 0u);
     }
   }
+  if (late && lane == 0) atomicCAS(a.status, 0, (int)QWM_ERR_TIMEOUT);
   if (bad) atomicCAS(a.status, 0, (int)QWM_ERR_NONFINITE);
   if (lane == 0) bulk_wait_all();
 }
@@ -408,9 +431,14 @@ __device__ __forceinline__ void st_chunk(uint8_t* base, int row, int ch, uint4 v
 struct DenseItem {
   int unit, lo, hi, slot;
 };
-// First of CTA b's key tiles among the tail's flattened tiles: tail_per each,
-// one more for the first tail_more CTAs.
+// First of CTA b's key tiles among the tail's flattened tiles: equal parts of
+// one query block per CTA (tail_parts > 0), or tail_per tiles each, one more for
+// the first tail_more CTAs, whatever block they fall in.
 __device__ __forceinline__ int64_t tail_start(const DenseArgs& a, int b) {
+  if (a.tail_parts > 0) {
+    const int k = b / a.tail_parts;
+    return (int64_t)k * a.NT + (int64_t)(b - k * a.tail_parts) * a.NT / a.tail_parts;
+  }
   return (int64_t)b * a.tail_per + min(b, a.tail_more);
 }
 // Items of CTA b in order: one whole query block per full wave, then its share
@@ -777,7 +805,8 @@ __global__ void __launch_bounds__(256) dense_combine(const DenseArgs a, int grid
   auto cta_of = [&](int64_t x) {
     return (int)(x < big ? x / (a.tail_per + 1) : a.tail_more + (x - big) / a.tail_per);
   };
-  const int b0 = cta_of(x0), b1 = cta_of(x1 - 1) + 1;
+  const int b0 = a.tail_parts > 0 ? k * a.tail_parts : cta_of(x0);
+  const int b1 = a.tail_parts > 0 ? b0 + a.tail_parts : cta_of(x1 - 1) + 1;
   pdl_wait();
   if (qi >= a.Nq || b1 == b0 + 1) return;
   const size_t base = (size_t)(2 * b0 + (tail_start(a, b0) < x0 ? 1 : 0)) * 256 + prow;   // part b0
@@ -813,6 +842,8 @@ __global__ void __launch_bounds__(256) dense_combine(const DenseArgs a, int grid
 }
 
 constexpr int kMinTail = 3;   // key tiles of a CTA's share of the tail, at least
+constexpr int kPartCost = 12;  // fixed time of a part (its Queries in, its partial results out and combined), in key tiles
+constexpr int kWholeCost = 4;  // of a whole block
 
 }  // namespace
 
@@ -825,11 +856,27 @@ DensePlan plan_dense(int64_t Nq, int heads, int64_t Nk, int nsm) {
   p.waves = (int)(units / nsm);
   p.n_tail = (int)(units - (int64_t)p.waves * nsm);
   const int64_t T = (int64_t)p.n_tail * p.NT;
-  int64_t g = (T + kMinTail - 1) / kMinTail;
-  if (g < p.n_tail) g = p.n_tail;
-  p.tail_ctas = (int)(g < nsm ? g : nsm);
-  p.tail_per = p.tail_ctas ? T / p.tail_ctas : 0;
-  p.tail_more = p.tail_ctas ? (int)(T % p.tail_ctas) : 0;
+  if (p.n_tail > 0) {
+    // Equal parts of each block, one per CTA, or the flattened tiles over every
+    // CTA: the latter leaves none idle, but most CTAs then run two parts.  48
+    // blocks of 110 tiles: 144 CTAs of 37 tiles 112 us a call, 152 of 35 126 us;
+    // 64 of 53: 87 and 93 us; 80 of 32: whole blocks 92, over every CTA 102 us;
+    // 80 of 272: 437 and 315 us.
+    int64_t s = nsm / p.n_tail, per = (p.NT + s - 1) / s;
+    if (per < kMinTail) per = kMinTail;
+    s = (p.NT + per - 1) / per;
+    int64_t g = (T + kMinTail - 1) / kMinTail;
+    if (g < p.n_tail) g = p.n_tail;
+    if (g > nsm) g = nsm;
+    if (per + (s > 1 ? kPartCost : kWholeCost) <= (T + g - 1) / g + 2 * kPartCost) {
+      p.tail_parts = (int)s;
+      p.tail_ctas = (int)(s * p.n_tail);
+    } else {
+      p.tail_ctas = (int)g;
+      p.tail_per = T / g;
+      p.tail_more = (int)(T % g);
+    }
+  }
   p.grid = p.waves > 0 ? nsm : p.tail_ctas;
   return p;
 }
@@ -847,6 +894,7 @@ cudaError_t launch_dense(const DenseArgs& a0, const AttendSlots& slots, const De
   a.waves = p.waves;
   a.n_tail = p.n_tail;
   a.tail_ctas = p.tail_ctas;
+  a.tail_parts = p.tail_parts;
   a.tail_per = p.tail_per;
   a.tail_more = p.tail_more;
   auto reb = a.L.sf ? (a.L.r == 0    ? rebuild_kernel<1, 0>
@@ -858,16 +906,16 @@ cudaError_t launch_dense(const DenseArgs& a0, const AttendSlots& slots, const De
                        : a.L.r == 16 ? rebuild_kernel<0, 16>
                                      : rebuild_kernel<0, 32>);
   const int n_units = slots.n + (a.Ncur > 0 ? 1 : 0);
-  // Tiles per CTA: U_r is staged once per CTA and each tile but the first is
-  // prefetched, so as many as leave two CTAs for every place on the GPU (two
-  // per SM), eight at most.  Wan-14B layer, per launch: 270 us with one, 193 us
-  // with eight.
+  // Tiles per CTA: U_r is staged once per CTA and each record but the first is
+  // copied a tile ahead, so as many as leave two CTAs for every place on the GPU
+  // (two per SM), eight at most.  Wan-14B layer, per launch: 205 us with one
+  // tile, 184 with two, 178 with four or eight; 84 tiles in all: 6.4 us with one
+  // each, 9.7 with two.
   const int64_t all = (int64_t)max_tiles * heads * n_units, per = all / (4 * p.nsm);
   const int tpc = per < 1 ? 1 : per > 8 ? 8 : (int)per;
-  constexpr int reb_smem = kRebThreads / 32 * kStage;
-  cudaError_t e = cudaFuncSetAttribute(reb, cudaFuncAttributeMaxDynamicSharedMemorySize, reb_smem);
+  cudaError_t e = cudaFuncSetAttribute(reb, cudaFuncAttributeMaxDynamicSharedMemorySize, kRebSmem);
   if (e != cudaSuccess) return e;
-  reb<<<dim3((unsigned)((max_tiles + tpc - 1) / tpc), (unsigned)heads, (unsigned)n_units), kRebThreads, reb_smem, st>>>(
+  reb<<<dim3((unsigned)((max_tiles + tpc - 1) / tpc), (unsigned)heads, (unsigned)n_units), kRebThreads, kRebSmem, st>>>(
       a, slots, tpc);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, D_SMEM)) != cudaSuccess)

@@ -190,7 +190,7 @@ struct DenseArgs {
   int32_t h0;                  // first head of the group
   // blocks of 256 queries of one head, numbered head by head: `waves` whole
   // ones per CTA, then n_tail ones whose key tiles are shared out over tail_ctas
-  int32_t bph, NT, waves, n_tail, tail_ctas, tail_more;
+  int32_t bph, NT, waves, n_tail, tail_ctas, tail_parts, tail_more;
   int64_t tail_per;            // tail key tiles of a CTA (one more for the first tail_more)
   uint8_t* img;                // [heads of the group][NT][K 32 KB | V 32 KB]
   float* part_o;               // [2 tail_ctas][256][128] fp32
@@ -198,7 +198,7 @@ struct DenseArgs {
   int64_t key0[kMaxSlots + 1]; // first key of each unit (cached chunks in order, then the active chunk)
 };
 struct DensePlan {
-  int32_t bph, NT, waves, n_tail, tail_ctas, tail_more, grid, nsm;
+  int32_t bph, NT, waves, n_tail, tail_ctas, tail_parts, tail_more, grid, nsm;
   int64_t tail_per;
 };
 DensePlan plan_dense(int64_t Nq, int heads, int64_t Nk, int nsm);
