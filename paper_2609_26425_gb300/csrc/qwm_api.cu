@@ -314,9 +314,20 @@ int device_sms() {
 }
 
 // Scratch of the path through operand images (attend_dense.cu): the heads are
-// taken in `groups` equal groups, each with its images and the partial results
-// of its split query blocks.
-constexpr size_t kDenseImages = (size_t)1 << 40;   // images of one group, at most (one head at least)
+// taken in equal groups, each with its images and the partial results of its
+// split query blocks.
+// A group's images take 2 GiB at most (one head at least), so that the scratch
+// of a long cache stays bounded (40 heads: one group up to 104 K keys); the
+// groups run one after another in the same buffer.
+constexpr size_t kDenseImages = (size_t)2 << 30;
+
+// Whether a call may take the images' path: its three launches take about 28 us
+// at the least, so not over few keys (400 keys in two units, 100 queries, 40
+// heads: 27.9 us against 22.5; 600 keys, 300 queries: 30.0 against 32.1), nor
+// over a single chunk below 1024, which the other kernel runs in one launch (880
+// keys and queries, 4 heads: 30.2 against 31.4; 640: 29.4 against 26.0; 4680,
+// 40 heads: 375 against 681).
+bool use_images(int units, int64_t Nk) { return Nk >= (units >= 2 ? 512 : 1024); }
 
 struct DenseGroups {
   int heads;        // of a group (the last may have fewer)
@@ -391,7 +402,7 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
   // follow where the running maximum and the binary16 probabilities are
   // rounded, which the other kernel's results fix.  The idle role of the
   // timeout test belongs to that kernel too.
-  if (workspace && units >= 2 && !lse && c->idle_role == 0) {
+  if (workspace && use_images(units, Nk) && !lse && c->idle_role == 0) {
     const DenseGroups g = dense_groups(Nq, c->L.H, Nk, nsm);
     if (workspace_bytes >= g.bytes) {
       qwm::DenseArgs d{};
@@ -467,10 +478,9 @@ size_t qwm_attend_workspace_bytes(const qwm_config* cfg, const qwm_cache* c, int
   int units = 0;
   int64_t longest = 0;
   const int64_t Nk = total_keys(c, N_cur, &units, &longest);
-  if (units < 2) return 0;
-  // enough for either path: which one runs depends on the call's lse
+  // enough for either path: which one runs depends on the call's lse too
   const size_t parts = qwm::attend_workspace_bytes(qwm::plan_attend(Nq, c->L.H, units, nsm, true));
-  const size_t dense = dense_groups(Nq, c->L.H, Nk, nsm).bytes;
+  const size_t dense = use_images(units, Nk) ? dense_groups(Nq, c->L.H, Nk, nsm).bytes : 0;
   return dense > parts ? dense : parts;
 }
 

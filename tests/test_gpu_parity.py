@@ -284,6 +284,34 @@ def test_fit_parity_full_size_sampled():
         assert np.array_equal(got[heads], ref["centroids"])
 
 
+@pytest.mark.parametrize("H,N,C,iters,kind", [
+    (1, 66000, 5, 2, "gauss"),     # token indices beyond 16 bits
+    (2, 3000, 100, 4, "tail"),     # clusters far above the average: members picked from the assignment
+    (12, 5000, 64, 2, "copies"),   # eight equal centroids a row: exact ties, the waiting list runs full
+    (1, 700, 64, 2, "few"),        # more tied centroids than a row may list: every centroid searched
+    (1, 300, 7, 3, "zero"),        # nothing but zeros
+])
+def test_fit_parity_lists_and_ties(H, N, C, iters, kind):
+    """The k-means paths that ordinary chunks rarely take, bit for bit."""
+    g = torch.Generator().manual_seed(N + C)
+    x = torch.randn(N, H, 128, generator=g)
+    if kind == "tail":
+        x[:, :, :4] *= 8.0 / torch.rand(N, H, 4, generator=g).clamp(min=1e-3)
+        x[: N // 2] *= 0.01
+    elif kind == "copies":
+        x = x[:8].repeat((N + 7) // 8, 1, 1)[:N]
+        x = x[torch.randperm(N, generator=g)]
+        x[(torch.arange(C) * N) // C] = x[(torch.arange(C) * N) // C % 8]
+    elif kind == "few":
+        x = x[torch.randint(0, 3, (N,), generator=g)]
+    elif kind == "zero":
+        x = torch.zeros(N, H, 128)
+    xt = x.to(torch.bfloat16).contiguous()
+    ref = orc.fit_centroids(synth.bits(xt), C, iters)
+    got = synth.bits(qwm.qwm_fit_centroids(qwm.config(H, C, kmeans_iters=iters), dev(xt)).cpu())
+    assert np.array_equal(got, ref["centroids"])
+
+
 def build_cache_and_reference(H, chunk_sizes, C, G, r, M, seed, *, Ncur, Nq, window=0, max_chunks=None,
                               psac_chunks=None, rows=None, scale_format=0):
     """Append chunks on the GPU and build the oracle's reference keys/values."""

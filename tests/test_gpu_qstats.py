@@ -115,6 +115,33 @@ def test_query_stats_parity(H, chunks, r):
     check_basis(st, q_all, r)
 
 
+@pytest.mark.parametrize("H,N,r,kind", [
+    (3, 1, 32, "gauss"),        # rank one: 127 equal eigenvalues
+    (2, 31, 32, "gauss"),       # rank below the vectors asked for
+    (2, 500, 32, "lowrank"),    # eight directions
+    (2, 400, 16, "dead"),       # half of the channels zero
+    (2, 400, 32, "twice"),      # every channel twice: half of the eigenvalues zero
+    (2, 300, 32, "graded"),     # scales over sixteen decades
+])
+def test_query_basis_special_spectra(H, N, r, kind):
+    """Repeated, zero and graded eigenvalues: the eigenvalues, and orthonormal
+    vectors that satisfy the eigen-equation."""
+    g = torch.Generator().manual_seed(N + r)
+    q = torch.randn(N, H, 128, generator=g)
+    if kind == "lowrank":
+        q = torch.einsum("nhk,hkc->nhc", torch.randn(N, H, 8, generator=g), torch.randn(H, 8, 128, generator=g))
+    elif kind == "dead":
+        q[:, :, ::2] = 0
+    elif kind == "twice":
+        q[:, :, 64:] = q[:, :, :64]
+    elif kind == "graded":
+        q *= 10.0 ** -(torch.arange(128) / 8.0)
+    q = q.to(torch.bfloat16).contiguous()
+    st = qwm.QueryStats(qwm.config(H, 64, psac_rank=r))
+    st.update(q.cuda())
+    check_basis(st, q, r)
+
+
 def test_query_stats_hadamard_closed_form():
     """Orthogonal +-1 rows scaled by n + 1 (and d - n): the sums are integers
     below 2^24 (exact in fp32), the eigenvalues are the squared scales and the
