@@ -53,12 +53,12 @@ def workload_numbers(wl, scale_format=0):
 
 
 def attend_traffic(workload):
-    """DRAM bytes per attend launch from the committed ncu summary, or None when
-    the kernel source has changed since those counters were taken or the
+    """DRAM bytes per attend call from the committed ncu summary, or None when
+    the kernels' source has changed since those counters were taken or the
     workload is not the one they were taken on."""
     import hashlib
-    prof = os.path.join(ROOT, "profiles", "attend_kernel_wan14b_layer.md")
-    src = os.path.join(ROOT, "paper_2609_26425_gb300", "csrc", "attend.cu")
+    prof = os.path.join(ROOT, "profiles", "attend_dense_wan14b_layer.md")
+    src = os.path.join(ROOT, "paper_2609_26425_gb300", "csrc", "attend_dense.cu")
     try:
         fields = {}
         with open(prof) as f:
@@ -343,21 +343,23 @@ def run_gpu(args, wl, rank, world):
         "append": {"ms": round(app_ms, 4), "gbs": round(app_gbs, 1),
                    "frac_of_measured_hbm": round(app_gbs / pk["hbm_gbs"], 4),
                    "algorithmic_bytes": nums["append_bytes"]},
-        "roofline": {"bound": "tensor", "kernel": "attend_kernel", "achieved": round(att_tflops, 2),
+        # the whole attend call: rebuild_kernel (keys to operand images) and dense_kernel
+        "roofline": {"bound": "tensor", "kernel": "rebuild_kernel + dense_kernel",
+                     "achieved": round(att_tflops, 2),
                      "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
                      "frac": round(att_tflops / pk["bf16_tflops"], 4), "traffic": attend_traffic(None if args.scale_format else wl.name),
                      "peak_src": pk["src"] + " burst bf16 (binary16 operands run at the bf16 rate)"},
         "e2e": {"value": round(e2e_value, 3), "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        # attend: one kernel; append: the candidate filter and the quantize kernel
-        # when M <= 8 and M < C, a single kernel otherwise
-        "gpu_launches": (1 + (2 if (M < C and M <= 8) else 1)) * args.steps,
+        # attend: the rebuild and the attention (the combine of split query blocks,
+        # where the plan has some, is not counted); append: one kernel
+        "gpu_launches": (2 + 1) * args.steps,
         "clocks": clk,
         "query_stats": {"update_ms": round(qs["update_ms"], 4),
                         "update_gbs": round(qs["update_bytes"] / (qs["update_ms"] * 1e-3) / 1e9, 1),
                         "update_frac_of_measured_hbm": round(
                             qs["update_bytes"] / (qs["update_ms"] * 1e-3) / 1e9 / pk["hbm_gbs"], 4),
                         "update_algorithmic_bytes": qs["update_bytes"],
-                        "basis_ms": round(qs["basis_ms"], 4), "jacobi_sweeps": qs["sweeps"],
+                        "basis_ms": round(qs["basis_ms"], 4), "solver_iterations": qs["sweeps"],
                         "l2": "update: 4 rotating copies of q (192 MB); basis: 256 MB flush before each launch"},
         # quality: share of queries whose highest-logit cached key moves away from the bf16 keys' one
         "top1_shift": shift,
@@ -590,10 +592,10 @@ def stack_line(args, wl, psac_rank=None):
                    "gbs": round(wl.layers * nums["append_bytes"] / (app_ms * 1e-3) / 1e9, 1),
                    "frac_of_measured_hbm": round(wl.layers * nums["append_bytes"] / (app_ms * 1e-3) / 1e9 /
                                                  pk["hbm_gbs"], 4)},
-        "roofline": {"bound": "tensor", "kernel": "attend_kernel", "achieved": round(tflops, 2),
+        "roofline": {"bound": "tensor", "kernel": "rebuild_kernel + dense_kernel", "achieved": round(tflops, 2),
                      "peak": pk["bf16_tflops"], "unit": "TFLOP/s", "frac": round(tflops / pk["bf16_tflops"], 4),
                      "traffic": None, "peak_src": pk["src"] + " burst bf16"},
-        "gpu_launches": (1 + 2) * wl.layers * len(rows),
+        "gpu_launches": (2 + 1) * wl.layers * len(rows),
         "clocks": clk, "per_step": rows,
     }
     if not args.no_cpu_baseline:

@@ -172,8 +172,9 @@ QWM_API qwm_status qwm_cache_set_idle_role(qwm_cache* cache, int32_t role);
 /* Scratch bytes qwm_fit_centroids needs for N tokens; 0 for an invalid
  * configuration.  With P = C rounded up to a multiple of 16 (at least 16),
  * each part padded to 256 bytes: a 256-byte status word, fp32 centroids
- * H*C*d*4, bf16 operand images H*P*512, norms H*P*4, H*4, counts and offsets
- * 2*H*C*4, assignment H*N and member lists H*N*4. */
+ * H*C*d*4, bf16 operand images H*P*512, norms H*P*4, exponents 2*H*4, counts
+ * 2*H*C*4 (one half of each reserved), assignment H*N, token norms H*N*4 and
+ * member lists H*N*4. */
 QWM_API size_t qwm_fit_workspace_bytes(const qwm_config* cfg, int64_t N);
 
 /* k-means centroids of one chunk, per head (Sec. 2: centroid-residual form of

@@ -774,7 +774,7 @@ size_t fit_workspace_bytes(int H, int d, int C, int64_t N) {
   b += (size_t)round_up((int64_t)H * Np * 512, 256);            // images
   b += (size_t)round_up((int64_t)H * Np * 4, 256);              // norms
   b += 2 * (size_t)round_up((int64_t)H * 4, 256);               // largest exponent (and a reserved field)
-  b += 2 * (size_t)round_up((int64_t)H * C * 4, 256);           // counts, offsets
+  b += 2 * (size_t)round_up((int64_t)H * C * 4, 256);           // counts (and a reserved field)
   b += (size_t)round_up((int64_t)H * N, 256);                   // assignment
   b += (size_t)round_up((int64_t)H * N * 4, 256);               // token norms
   b += (size_t)round_up((int64_t)H * N * 4, 256);               // member lists
@@ -913,8 +913,8 @@ extern "C" QWM_API qwm_status qwm_fit_centroids_noalloc(const qwm_config* cfg, c
   a.x = static_cast<const __nv_bfloat16*>(x);
   a.out = static_cast<__nv_bfloat16*>(centroids);
   fit_carve(a, ws);
-  // launch_fit clears the status word, the counts and the largest norms and
-  // writes every centroid, image and norm before reading it, so nothing
+  // launch_fit clears the status word, the counts and the largest exponents
+  // and writes every centroid, image and norm before reading it, so nothing
   // depends on what an earlier call left in the array.
   return launch_fit(a, static_cast<cudaStream_t>(stream)) == cudaSuccess ? QWM_OK : QWM_ERR_CUDA;
 }
