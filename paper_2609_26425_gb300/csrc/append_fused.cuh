@@ -155,7 +155,24 @@ inline int fused_shares(FusedShares& sh, int units, int tiles, int ctas, int kco
     if (fill(mid) <= ctas) hi = mid;
     else lo = mid + 1;
   }
-  return fill(hi);
+  // CTAs left over take halves of the largest small shares: two groups at work
+  // share an SM's issue slots, and a tile takes longer than alone (12 heads, 880
+  // tokens, 168 units: r = 8, 96 CTAs 39.5 us, 152 CTAs 31.3; r = 32, 59.5 and 49.9).
+  int used = fill(hi);
+  for (int n = 8; n >= 2 && used < ctas; --n) {
+    FusedShares f = sh;
+    int out = 0, spare = ctas - used;
+    for (int b = 0; b < used; ++b) {
+      sh.first[out++] = f.first[b];
+      if (spare > 0 && f.first[b + 1] - f.first[b] == n) {
+        sh.first[out++] = f.first[b] + (n / 2 + 1) / 2 * 2 - (n == 2);
+        --spare;
+      }
+    }
+    used = out;
+    for (int e = used; e <= ctas; ++e) sh.first[e] = units;
+  }
+  return used;
 }
 
 // CAPT = M + 1 (the ranked list of a row; kMaxFilterM + 1 for the candidate
