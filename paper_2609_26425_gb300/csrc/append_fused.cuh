@@ -116,7 +116,8 @@ struct FusedShares {
 // taking kSetup and the tiles of the group that has more of them.  A Key tile
 // costs more than a Value tile, and with equal shares the CTAs on Values idled
 // for the difference.  The time is found by trials, each CTA in turn taking
-// what fits in it (host arithmetic, about 250 steps a trial, fewer than ten).
+// what fits in it (host arithmetic: a step per run and trial, fewer than ten
+// trials; with a step per CTA a call took 4 to 20 us more on the host).
 inline int fused_shares(FusedShares& sh, int units, int tiles, int ctas, int kcost, int vcost) {
   constexpr int64_t kSetup = 5;
   const int nkey = units / 2;
@@ -138,6 +139,25 @@ inline int fused_shares(FusedShares& sh, int units, int tiles, int ctas, int kco
     for (int e = b; e <= ctas; ++e) sh.first[e] = units;
     return b;
   };
+  // the CTAs that fill() would use, run by run
+  auto count = [&](int64_t limit) -> int64_t {
+    int64_t b = 0, used = limit;   // no CTA begun
+    for (int u = 0; u < units; u += tiles) {
+      const int64_t c = u < nkey ? kcost : vcost, full = (limit - kSetup) / c;
+      int64_t rest = tiles;
+      if (limit - used >= kSetup + c) {
+        const int64_t room = 2 * ((limit - used - kSetup) / c), take = rest < room ? rest : room;
+        used += kSetup + (take + 1) / 2 * c;
+        rest -= take;
+      }
+      if (rest > 0) {
+        const int64_t n = rest / (2 * full), left = rest - n * 2 * full;
+        b += n + (left > 0);
+        used = kSetup + (left > 0 ? (left + 1) / 2 : full) * c;
+      }
+    }
+    return b;
+  };
   // one unit per CTA always fits in a Key tile's time when the CTAs suffice
   if (units <= ctas) {
     for (int b = 0; b <= ctas; ++b) sh.first[b] = b < units ? b : units;
@@ -146,20 +166,22 @@ inline int fused_shares(FusedShares& sh, int units, int tiles, int ctas, int kco
   // from the mean share of a group upwards, to within 1 %
   const int64_t most = kSetup + (kcost > vcost ? kcost : vcost), mean = (int64_t)nkey * (kcost + vcost) / (2 * ctas);
   int64_t lo = mean > most ? mean : most, hi = lo;
-  while (fill(hi) > ctas) {
+  while (count(hi) > ctas) {
     lo = hi + 1;
     hi += hi / 16 + 1;
   }
   while (hi - lo > hi / 128) {
     const int64_t mid = (lo + hi) / 2;
-    if (fill(mid) <= ctas) hi = mid;
+    if (count(mid) <= ctas) hi = mid;
     else lo = mid + 1;
   }
   // CTAs left over take halves of the largest small shares: two groups at work
   // share an SM's issue slots, and a tile takes longer than alone (12 heads, 880
   // tokens, 168 units: r = 8, 96 CTAs 39.5 us, 152 CTAs 31.3; r = 32, 59.5 and 49.9).
-  int used = fill(hi);
-  for (int n = 8; n >= 2 && used < ctas; --n) {
+  int used = fill(hi), big = 1;
+  for (int b = 0; b < used && used < ctas; ++b)
+    if (sh.first[b + 1] - sh.first[b] > big) big = sh.first[b + 1] - sh.first[b];
+  for (int n = big < 8 ? big : 8; n >= 2 && used < ctas; --n) {
     FusedShares f = sh;
     int out = 0, spare = ctas - used;
     for (int b = 0; b < used; ++b) {
