@@ -26,7 +26,8 @@
 //     squared, d = |x|^2 - 2 s_k the distance found (+ E): so every j with
 //     s_j > s_k - c (|x|^2 + 2.02 (|x|^2 + d)) is a candidate for the exact
 //     argmin.  A row with a single candidate is decided, the others are
-//     rescored with the sequential fp32 distance.
+//     rescored with the sequential fp32 distance.  Columns past C hold -inf;
+//     heads with values from 2^59 up are not screened (kMaxExp).
 //   fit_means   (four warps per centroid): exact member sums (bf16 values of
 //     ordinary range add exactly, so the order does not matter) from the list of
 //     members that the assignment leaves per centroid, the mean, and the next
@@ -63,7 +64,14 @@ constexpr int A_CND = A_CNT + 4 * AT * 4;     // [128][4 quarters][kRowCap] cand
 constexpr int A_BAR = A_CND + AT * 4 * kRowCap;   // mbarriers, pair counter, flag, TMEM slot
 constexpr int A_SMEM = A_BAR + 128 + 1024;
 static_assert(A_SMEM <= 232448, "shared memory of the assignment kernel");
-constexpr uint32_t kPadNorm = 0x0000F149u;    // bf16 -1e30 | 0 << 16: a padding column never wins
+constexpr uint32_t kPadNorm = 0x0000FF80u;    // bf16 -inf | 0 << 16: a padding column never wins, whatever the data
+// The screening holds where no product, norm or sum of it leaves the fp32
+// range: token values below 2^59 (this bf16 exponent field), so that |x|^2 and
+// |mu|^2 stay below 2^125.  A head with a larger value, an infinity or a NaN
+// among its tokens has every row searched centroid by centroid: there a
+// centroid may be inf or NaN, which the sequential search orders as the
+// definition does (a NaN never replaces a distance, and centroid 0's is kept).
+constexpr int kMaxExp = 185;
 
 // Operand block of rows of 16 two-byte values without swizzle: 8 rows x 16
 // bytes contiguous, the second half of the values 128 bytes on, row groups 256
@@ -397,6 +405,7 @@ __global__ void __launch_bounds__(ANT, 1)
       const int64_t n = (int64_t)tile * 128 + row;
       const bool valid = n < a.N;
       const float kx = valid ? a.xn2[(size_t)h * a.N + n] : 0.0f;
+      const bool in_range = a.emax[h] <= kMaxExp;
       const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar_mma(b), (t >> 1) & 1));
       tc_fence_after();
       // s_j of this quarter's columns and the largest
@@ -420,7 +429,7 @@ __global__ void __launch_bounds__(ANT, 1)
       mx = fmaxf(fmaxf(sMin[row], sMin[AT + row]), fmaxf(sMin[2 * AT + row], sMin[3 * AT + row]));
       const float dist = fmaxf(fmaf(-2.0f, mx, kx), 0.0f);
       const float thr = fmaf(-kC, fmaf(2.02f, kx + dist, kx), mx) - 1e-30f;
-      const bool fin = ok && thr > -INFINITY && thr < INFINITY && kx < INFINITY;
+      const bool fin = ok && in_range && thr > -INFINITY && thr < INFINITY;
       // this quarter's candidates, ascending (bit 31 - e of a mask: column e)
       int cnt = 0;
       uint32_t word = 0xFFu;   // count (0xFF: every centroid), first candidate << 8

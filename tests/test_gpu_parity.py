@@ -312,6 +312,31 @@ def test_fit_parity_lists_and_ties(H, N, C, iters, kind):
     assert np.array_equal(got, ref["centroids"])
 
 
+@pytest.mark.parametrize("C", [4, 31, 63, 250, 255])   # one to eight padding columns, and many
+@pytest.mark.parametrize("kind", ["1e13", "1e15", "1e17", "1e30", "mixed", "nan0", "nan", "inf"])
+def test_fit_parity_extreme_values(C, kind):
+    """Values at which every real centroid scores far below an ordinary one's
+    range (large rows, and small rows among large initial centroids), and heads
+    with a NaN or an infinity among their tokens: the same centroids as the
+    definition's, NaN for NaN, and the finite head beside them untouched."""
+    H, N, iters = 3, 700, 3
+    g = torch.Generator().manual_seed(C)
+    x = torch.randn(N, H, 128, generator=g)
+    if kind == "mixed":              # the strided tokens are large, all others near zero
+        far = (torch.arange(C) * N) // C
+        x *= 1e-3
+        x[far] = torch.randn(C, H, 128, generator=g) * 4e15
+    elif kind in ("nan0", "nan", "inf"):
+        x[0 if kind == "nan0" else 333, 1, 5] = float("inf") if kind == "inf" else float("nan")
+    else:
+        x *= float(kind)
+    xt = x.to(torch.bfloat16).contiguous()
+    ref = synth.from_bits(orc.fit_centroids(synth.bits(xt), C, iters)["centroids"]).float()
+    got = qwm.qwm_fit_centroids(qwm.config(H, C, kmeans_iters=iters), dev(xt)).float().cpu()
+    assert torch.equal(torch.isnan(got), torch.isnan(ref))
+    assert torch.equal(torch.where(torch.isnan(got), 0.0, got), torch.where(torch.isnan(ref), 0.0, ref))
+
+
 def build_cache_and_reference(H, chunk_sizes, C, G, r, M, seed, *, Ncur, Nq, window=0, max_chunks=None,
                               psac_chunks=None, rows=None, scale_format=0):
     """Append chunks on the GPU and build the oracle's reference keys/values."""
