@@ -101,12 +101,14 @@ __device__ __forceinline__ int sw_off(int rows, int row, int ch) {
 
 // The sequential fp32 distance of the definition: channel order, the
 // difference, its square and the running sum each rounded on its own.
-// (One thread: for rows left to the search of every centroid.)
+// (One thread: for rows left to the search of every centroid.  mu is read by
+// ordinary loads: fit_means may still be writing it when the assignment's
+// launch starts, so it is no read-only data of that kernel.)
 __device__ __noinline__ float exact_dist(const __nv_bfloat16* x, const float* mu) {
   float acc = 0.0f;
 #pragma unroll 1
   for (int ch = 0; ch < 16; ++ch) {
-    const float4 ma = __ldg(reinterpret_cast<const float4*>(mu) + 2 * ch), mb = __ldg(reinterpret_cast<const float4*>(mu) + 2 * ch + 1);
+    const float4 ma = reinterpret_cast<const float4*>(mu)[2 * ch], mb = reinterpret_cast<const float4*>(mu)[2 * ch + 1];
     const uint4 xr = __ldg(reinterpret_cast<const uint4*>(x) + ch);
     const uint32_t xw[4] = {xr.x, xr.y, xr.z, xr.w};
     const float ms[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
@@ -128,7 +130,7 @@ __device__ __noinline__ float2 exact_dist2(uint2 xv, const float* mu0, const flo
   const int lane = threadIdx.x & 31;
   const float xf[4] = {__uint_as_float(xv.x << 16), __uint_as_float(xv.x & 0xFFFF0000u), __uint_as_float(xv.y << 16),
                        __uint_as_float(xv.y & 0xFFFF0000u)};
-  const float4 ma = __ldg(reinterpret_cast<const float4*>(mu0) + lane), mb = __ldg(reinterpret_cast<const float4*>(mu1) + lane);
+  const float4 ma = reinterpret_cast<const float4*>(mu0)[lane], mb = reinterpret_cast<const float4*>(mu1)[lane];
   const float m0[4] = {ma.x, ma.y, ma.z, ma.w}, m1[4] = {mb.x, mb.y, mb.z, mb.w};
   float s0[4], s1[4], d0 = 0.0f, d1 = 0.0f;
 #pragma unroll
