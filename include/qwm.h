@@ -164,7 +164,9 @@ QWM_API qwm_status qwm_cache_set_wait_limit(qwm_cache* cache, uint64_t ns);
  * QWM_ROLE_V_REBUILD, the attention calls made afterwards leave the role that
  * rebuilds V_hat idle, so the MMA warp's bounded wait for its first tile runs
  * out (with a short qwm_cache_set_wait_limit, in milliseconds) and the call
- * records QWM_ERR_TIMEOUT instead of computing.  0 restores normal work; any
+ * records QWM_ERR_TIMEOUT instead of computing.  A call through the scratch's
+ * operand images fetches no packed record and publishes no Value image: the
+ * rebuild's wait for its record runs out as well.  0 restores normal work; any
  * other role returns QWM_ERR_INVALID_ARG. */
 #define QWM_ROLE_V_REBUILD 1
 QWM_API qwm_status qwm_cache_set_idle_role(qwm_cache* cache, int32_t role);

@@ -302,7 +302,10 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
   bool bad = false;
   // The packed records come by bulk copies, a tile ahead: read from global
   // memory in the warps, their latency (twice a tile) bound the kernel.
+  int fetched = 0;   // copies issued (thread 0); none under the test hook's idle role
   auto fetch = [&](int tl) {
+    if (a.idle_role == QWM_ROLE_V_REBUILD) return;
+    ++fetched;
     const int b = (tl - tl0) & 1;
     mbar_arrive_expect_tx(smem_u32(s_bar + b), (uint32_t)L.tile_bytes);
     bulk_g2s(smem_u32(s_rec + b * kRecord), hb + L.tiles_off + (int64_t)tl * L.tile_bytes, (uint32_t)L.tile_bytes,
@@ -333,6 +336,7 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
   }
   const int r0 = (warp & 3) * 32;        // this warp's rows of each tile
   bool late = false;                     // a wait ran out (what follows is not used, but stays in bounds: id 0)
+  bool stop = false;                     // some warp's wait ran out: tiles were left
   for (int tl = tl0; tl < tl1; ++tl) {
     const int nv = min(128, ntok - tl * 128);
     const int64_t key0 = a.key0[u] + tl * 128;     // the tile's first key among the packed keys
@@ -367,7 +371,10 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
     }
     uint4 pm = make_uint4(0u, 0u, 0u, 0u);
     if (psac && key) pm = ldg16(hb + L.pmask + (int64_t)tl * 16);
-    __syncthreads();   // U_r and the barriers are in place; every warp is done with the record before
+    // U_r and the barriers are in place; every warp is done with the record
+    // before; nothing more is fetched once a wait has run out
+    if (tl == tl0) __syncthreads();
+    else if ((stop = __syncthreads_or(late))) break;
     if (tid == 0 && tl + 1 < tl1) fetch(tl + 1);
     if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(s_bar + ((tl - tl0) & 1)), ((tl - tl0) >> 1) & 1, a.wait_ns))) late = true;
     const uint8_t* tb = s_rec + ((tl - tl0) & 1) * kRecord;
@@ -405,6 +412,10 @@ __global__ void __launch_bounds__(kRebThreads, 2) rebuild_kernel(const DenseArgs
   if (late && lane == 0) atomicCAS(a.status, 0, (int)QWM_ERR_TIMEOUT);
   if (bad) atomicCAS(a.status, 0, (int)QWM_ERR_NONFINITE);
   if (lane == 0) bulk_wait_all();
+  // records still under way (a wait ran out) land before the CTA's memory goes away
+  if (late || stop)
+    for (int k = fetched > 2 ? fetched - 2 : 0; k < fetched; ++k)
+      mbar_wait(smem_u32(s_bar + (k & 1)), (k >> 1) & 1, a.wait_ns);
 }
 
 // ------------------------------------------------------------------ attention
@@ -762,6 +773,10 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const DenseArgs a) 
       while (ok && items.next(a, it)) {
         const uint8_t* src = a.img + ((size_t)(it.unit / a.bph) * a.NT + it.lo) * kImgTile;
         for (int j = 0; j < 2 * (it.hi - it.lo); ++j, ++n) {
+          if ((j & 1) && a.idle_role == QWM_ROLE_V_REBUILD) {   // test hook: no Value image is published
+            ok = false;
+            break;
+          }
           const int s = (int)(n % kStages);
           if (n >= kStages && !mbar_wait(bar(B_EMPTY + s), ((n / kStages) - 1) & 1, a.wait_ns)) {
             ok = false;

@@ -403,9 +403,8 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
   const int64_t Nk = total_keys(c, N_cur, &units, &longest);
   // The images' path gives no log-sum-exp: that is fp32, and its last digits
   // follow where the running maximum and the binary16 probabilities are
-  // rounded, which the other kernel's results fix.  The idle role of the
-  // timeout test belongs to that kernel too.
-  if (workspace && use_images(units, Nk) && !lse && c->idle_role == 0) {
+  // rounded, which the other kernel's results fix.
+  if (workspace && use_images(units, Nk) && !lse) {
     const DenseGroups g = dense_groups(Nq, c->L.H, Nk, nsm);
     if (workspace_bytes >= g.bytes) {
       qwm::DenseArgs d{};
@@ -421,6 +420,7 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
       d.sm_scale = sm_scale;
       d.out = static_cast<__nv_bfloat16*>(out);
       d.wait_ns = c->wait_ns;
+      d.idle_role = c->idle_role;
       d.img = static_cast<uint8_t*>(workspace);
       d.part_o = reinterpret_cast<float*>(d.img + g.images);
       int64_t key = 0;

@@ -187,6 +187,7 @@ struct DenseArgs {
   float sm_scale;
   __nv_bfloat16* out;          // [Nq][H][d]
   uint64_t wait_ns;            // limit of every bounded wait
+  int32_t idle_role;           // QWM_ROLE_*: a role that publishes nothing (test hook), 0 = none
   int32_t h0;                  // first head of the group
   // blocks of 256 queries of one head, numbered head by head: `waves` whole
   // ones per CTA, then n_tail ones whose key tiles are shared out over tail_ctas

@@ -63,3 +63,40 @@ def test_attend_wait_that_runs_out_records_timeout_and_next_call_is_exact():
     V = np.concatenate([V, orc.bf16_to_f32(vb[:100]).astype(np.float64)])
     ref, _ = orc.attend(synth.bits(q), K, V, 1 / math.sqrt(128))
     compare_attention(out.float().cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("N,Ncur", [(1100, 100), (700, 0)])   # a rebuilt and an active unit; the rebuilt chunks alone
+def test_attend_images_wait_that_runs_out_records_timeout_and_next_call_is_the_same(N, Ncur):
+    """The calls that go through the scratch's operand images: no packed record
+    and no Value image is published, so the waits of the rebuild and of the
+    attention kernel run out; both end by themselves and the next ordinary call
+    with the same scratch gives the same bits as before."""
+    H, C, r = 2, 16, 16
+    q, k, v = (synth.gaussian_bf16(61 + i, N, H, 128) for i in range(3))
+    kb, vb = synth.bits(k), synth.bits(v)
+    kc, vc = (dev(synth.from_bits(strided_centroids(b, C))) for b in (kb, vb))
+    cfg = qwm.config(H, C, psac_rank=r)
+    cache = qwm.Cache(cfg, N, 2)
+    for _ in range(2):
+        qwm.qwm_quantize_append(cfg, cache, dev(k), dev(v), kc, vc, U=dev(synth.random_orthonormal(64, H, 128, r)))
+    qd, cur = dev(q), (dev(k[:Ncur]), dev(v[:Ncur])) if Ncur else (None, None)
+    ws = qwm.attend_workspace(cfg, cache, N, Ncur)
+    keys = 2 * N + Ncur
+    assert ws.numel() >= H * (keys + 127) // 128 * 65536   # room for the images: their path runs
+    out = qwm.qwm_attend(cfg, cache, qd, *cur, workspace=ws)
+    assert cache.status() == 0
+    cache.set_wait_limit(1_000_000)            # 1 ms
+    cache.set_idle_role(qwm.QWM_ROLE_V_REBUILD)
+    scratch = torch.empty_like(out)
+    t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    t0.record()
+    qwm.qwm_attend(cfg, cache, qd, *cur, out=scratch, workspace=ws)
+    t1.record()
+    torch.cuda.synchronize()                   # the kernels end by themselves
+    assert cache.status() == TIMEOUT
+    assert t0.elapsed_time(t1) < 500.0         # a few limits, not the default one of 2 s
+    cache.set_idle_role(0)
+    cache.set_wait_limit(2_000_000_000)
+    again = qwm.qwm_attend(cfg, cache, qd, *cur, workspace=ws)
+    assert cache.status() == 0
+    assert torch.equal(again, out)
