@@ -283,9 +283,11 @@ __global__ void __launch_bounds__(ANT, 1)
     const uint32_t id = idesc_f16(128, Nm, false, true);
     const uint32_t aI = smem_u32(sm + A_IMG);
     int cur_h = -1;
-    uint32_t ph_img = 0;
+    uint32_t images = 0;       // heads' images loaded
     bool go = true;
+    int loads = 0, mmas = 0;   // tiles loaded, tiles multiplied
     auto load_tile = [&](int t) {
+      ++loads;
       const int u = u0 + t, h = u / tiles, b = t & 1;
       const uint32_t aX = smem_u32(sm + A_X + b * 32768);
       if (lane == 0) {
@@ -310,19 +312,15 @@ __global__ void __launch_bounds__(ANT, 1)
           for (int j = lane; j < Npad; j += 32)
             *reinterpret_cast<uint32_t*>(sm + A_NRM + k16_off(j)) = a.nrm[(size_t)h * Npad + j];
           fence_proxy_async_smem();
-          go = mbar_wait(bar_img, ph_img);
-          ph_img ^= 1;
+          go = mbar_wait(bar_img, images & 1);
+          ++images;
           cur_h = h;
         }
       }
       go = go && mbar_wait(bar_tma(b), (t >> 1) & 1);
       go = go && (t < 2 || mbar_wait(bar_free(b), ((t >> 1) - 1) & 1));
       go = __all_sync(0xFFFFFFFFu, go);
-      if (!go) {
-        mbar_wait(bar_tma(b), (t >> 1) & 1);   // no copy outlives the CTA
-        *s_err = 1;
-        break;
-      }
+      if (!go) break;
       tc_fence_after();
       if (lane == 0) {
         const uint32_t aX = smem_u32(sm + A_X + b * 32768);
@@ -338,17 +336,20 @@ __global__ void __launch_bounds__(ANT, 1)
         umma_ss(tD, desc_k16(smem_u32(sm + A_ONE)), desc_k16(smem_u32(sm + A_NRM)), id, 1u);
         umma_commit(bar_mma(b));
       }
+      ++mmas;
       __syncwarp();
       // the next tile's copy, once the MMAs of the tile before this one have left its buffer
       if (t + 1 < T) {
         if (t >= 1) go = __all_sync(0xFFFFFFFFu, mbar_wait(bar_mma(b ^ 1), ((t - 1) >> 1) & 1));
-        if (!go) {
-          *s_err = 1;
-          break;
-        }
+        if (!go) break;
         load_tile(t + 1);
       }
     }
+    if (!go) *s_err = 1;
+    // no copy and no MMA outlives the CTA's memory, also where a wait ran out
+    if (loads) mbar_wait(bar_tma((loads - 1) & 1), ((loads - 1) >> 1) & 1);
+    if (images) mbar_wait(bar_img, (images - 1) & 1);
+    if (mmas) mbar_wait(bar_mma((mmas - 1) & 1), ((mmas - 1) >> 1) & 1);
   } else {
     // ---------------- epilogue: warps 0-15
     const int qt = warp >> 2, row = (warp & 3) * 32 + lane;
