@@ -516,21 +516,27 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
   hi = hi * scale + 1e-6f;
   __syncthreads();
 
-  // ---- eigenvalues: counts at a grid of points, then each one's interval in
-  // sections, a point per thread: all 128 (four threads each) when they are
-  // asked for, else the r largest by 128 threads (a warp per sub-partition:
-  // the counts of 16 warps are bound by issue, those of four by latency)
+  // ---- eigenvalues: counts at a grid of 128 points, then each one's interval
+  // in sections, a point per thread.  The leading ones (r of them at least) by
+  // threads 0 .. 127, the others, when they are asked for, by two threads each
+  // of the warps after them: the leading ones, which the vectors' solves are
+  // shifted by, are the same bits either way.  (A warp per sub-partition for
+  // the leading ones: the counts of 16 warps are bound by issue, those of four
+  // by latency.)
   {
     const float* d = js + Q_D;
     const float* e2 = js + Q_E2;
     int* gc = reinterpret_cast<int*>(js + Q_CNT);
-    const int np = evals ? 512 : 128;                       // threads at work, and grid points
-    const int per = evals ? 4 : r > 16 ? 4 : r > 8 ? 8 : 16;  // threads per eigenvalue
+    constexpr int np = 128;                                  // grid points
+    const int lper = r > 16 ? 4 : r > 8 ? 8 : 16;            // threads per leading eigenvalue
+    const int nlead = 128 / lper;
     const float st = (hi - lo) / (float)(np + 1);
     if (tid < np) gc[tid] = sturm_count(d, e2, fmaf(st, (float)(tid + 1), lo));
     __syncthreads();
-    if (tid < np) {
-      const int ev = tid / per, q = tid & (per - 1);
+    if (tid < 128 || (evals && warp < 4 + (2 * (128 - nlead) + 31) / 32)) {
+      const int per = tid < 128 ? lper : 2;
+      const int own = tid < 128 ? tid / lper : nlead + (tid - 128) / 2;
+      const int ev = min(own, 127), q = tid & (per - 1);     // past the last one (in whole warps): its copies
       const int idx = 127 - ev;   // eigenvalue ev of the decreasing order is number idx of the increasing one
       int g0 = 0, g1 = np;        // first grid point with more than idx eigenvalues below it
       while (g0 < g1) {
@@ -540,8 +546,8 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
       }
       float l = g0 == 0 ? lo : fmaf(st, (float)g0, lo), u = g0 == np ? hi : fmaf(st, (float)(g0 + 1), lo);
       const float part = 1.0f / (float)(per + 1);
-      // until the interval is below 2^-24: 2 / 513 / 5^7, 2 / 129 / 5^8, 9^6, 17^5
-      const int rounds = evals ? 7 : per == 4 ? 8 : per == 8 ? 6 : 5;
+      // until the interval is below 2^-24: 2 / 129 / 3^12, 5^8, 9^6, 17^5
+      const int rounds = per == 2 ? 12 : per == 4 ? 8 : per == 8 ? 6 : 5;
 #pragma unroll 1
       for (int it = 0; it < rounds; ++it) {
         const float wd = (u - l) * part;
@@ -553,7 +559,7 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
         u = first == per ? u : fmaf(wd, (float)(first + 1), l);
         l = nl;
       }
-      if (q == 0) js[Q_LAM + ev] = 0.5f * (l + u);
+      if (q == 0 && own == ev) js[Q_LAM + ev] = 0.5f * (l + u);
     }
   }
   __syncthreads();

@@ -259,3 +259,17 @@ def test_query_stats_full_size_sampled():
     heads = [0, 17, 39]
     check_sums(st, q_all, heads)
     check_basis(st, q_all, r, heads)
+
+
+@pytest.mark.parametrize("H,N,r", [(4, 880, 8), (3, 500, 16), (2, 1000, 32), (2, 31, 32), (40, 4680, 16)])
+def test_query_basis_is_the_same_without_eigenvalues(H, N, r):
+    """U and w do not depend on what else is asked for: the same bits without
+    the eigenvalues, and the eigenvalues alone are those given with U."""
+    q = workload_queries("wan14b_layer", 0, tokens=N, heads=H).cuda()
+    st = qwm.QueryStats(qwm.config(H, 64, psac_rank=r))
+    st.update(q)
+    w, U, lam = st.basis(w=True, U=True, eigenvalues=True)
+    w1, U1, _ = st.basis(w=True, U=True)
+    _, _, lam1 = st.basis(w=False, U=False, eigenvalues=True)
+    assert st.read() == (0, N)
+    assert torch.equal(w, w1) and torch.equal(U.view(torch.int16), U1.view(torch.int16)) and torch.equal(lam, lam1)
