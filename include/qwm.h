@@ -301,7 +301,8 @@ QWM_API qwm_status qwm_attend_ws(const qwm_config* cfg, const qwm_cache* cache, 
  * qwm_query_stats_bytes(cfg) bytes, 256-byte aligned:
  *   byte 0    int32 device status word (QWM_OK or the first kernel error)
  *   byte 8    uint64 Query count N_<t (tokens folded in so far)
- *   byte 16   int32 iterations of qwm_query_basis's eigen-solver (maximum over heads)
+ *   byte 16   int32 steps of qwm_query_basis's inverse iteration since the reset
+ *             (maximum over heads and calls; 1: none needed, 30: not converged)
  *   byte 256  fp32 sums S_h = sum over past Queries of q q^T, [H][d][d] row-major.
  * --------------------------------------------------------------------------- */
 
@@ -329,8 +330,9 @@ QWM_API qwm_status qwm_query_stats_update(const qwm_config* cfg, void* stats, co
  *   eigenvalues: fp32 [H][d], all eigenvalues of M_h in decreasing order.
  * Any of w, U, eigenvalues may be NULL.  The eigen-solver works in fp32 on the
  * whole 128 x 128 matrix: Householder tridiagonalisation, multisection and
- * inverse iteration; a matrix with no off-diagonal entry above 2^-20 of the
- * Frobenius norm counts as diagonal. */
+ * inverse iteration until every vector's residual is below 2^-17 of the norm
+ * (two steps at least, 30 at most); a matrix with no off-diagonal entry above
+ * 2^-20 of the Frobenius norm counts as diagonal. */
 QWM_API qwm_status qwm_query_basis(const qwm_config* cfg, const void* stats, float* w, void* U, float* eigenvalues,
                                    void* stream);
 

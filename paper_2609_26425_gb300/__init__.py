@@ -467,7 +467,8 @@ class QueryStats:
         return st.value, cnt.value
 
     def sweeps(self) -> int:
-        """Iterations of the basis computation's eigen-solver (maximum over heads)."""
+        """Steps of the basis computation's inverse iteration since the reset
+        (maximum over heads and calls; 1: none needed, 30: not converged)."""
         return int(self.buffer[16:20].view(torch.int32).item())
 
 

@@ -24,7 +24,7 @@ namespace qwm {
 namespace {
 using namespace ptx;
 
-constexpr int kStatsHeader = 256;   // status word, count, sweeps; then the sums
+constexpr int kStatsHeader = 256;   // status word, count, solver steps; then the sums
 
 // ------------------------------------------------------------------ Gram sums
 constexpr int kGTok = 64;                        // tokens per stage
@@ -194,7 +194,9 @@ constexpr int Q_RED = Q_XB + 256;                // [32]
 constexpr int Q_CNT = Q_RED + 32;                // counts at the grid points [512]
 constexpr int Q_ORD = Q_CNT + 512;               // order of a diagonal matrix [128]
 constexpr int kBasisSmem = (Q_ORD + 128) * 4;
-constexpr int kIter = 2;                         // steps of inverse iteration
+constexpr int kIter = 2;                         // steps of inverse iteration, at least
+constexpr int kMaxIter = 30;                     // at most (a basis that took as many has not converged)
+constexpr float kResidual = 7.6293945e-6f;       // 2^-17 of the norm: largest entry of T y - lambda y
 constexpr float kTinyPivot = 1.1920929e-7f;      // 2^-23 of the matrix norm
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -244,11 +246,11 @@ __device__ __forceinline__ int sturm_count(const float* d, const float* e2, floa
 // w from the diagonal of S (Eq. 8) and the leading eigenvectors of M = S /
 // count (Eq. 15), one CTA per head: Householder tridiagonalisation with M in
 // registers (thread = 4 rows x 8 columns), eigenvalues by multisection on
-// Sturm counts, the r leading vectors by two steps of inverse iteration from
-// fixed pseudo-random vectors (LU with partial pivoting, a thread per vector),
-// each followed by modified Gram-Schmidt in decreasing order (so equal
-// eigenvalues get an orthonormal basis), and the Householder vectors applied
-// back.  A matrix whose off-diagonal entries are all below 2^-20 of its norm
+// Sturm counts, the r leading vectors by inverse iteration from fixed
+// pseudo-random vectors (LU with partial pivoting, a thread per vector; two
+// steps, and more while a residual is above 2^-17 of the norm), each step
+// followed by modified Gram-Schmidt in decreasing order (so equal eigenvalues
+// get an orthonormal basis), and the Householder vectors applied back.  A matrix whose off-diagonal entries are all below 2^-20 of its norm
 // counts as diagonal.
 // Bound by the latency of its serial chain: at 40 heads 126 reduction steps of
 // 1.7 K cycles (214 K), multisection 42 K, LU 11 K, inverse iteration and
@@ -256,7 +258,8 @@ __device__ __forceinline__ int sturm_count(const float* d, const float* e2, floa
 // quarter of its columns per thread a step took 2.1 K cycles: every thread then
 // read 32 values of v and of p from shared memory, 1 K cycles of its bandwidth.
 // Statistics reset, update and basis of the Wan-14B layer: 884 us with cyclic
-// Jacobi (7 sweeps of 127 rounds of 2 K cycles), 189 us.
+// Jacobi (7 sweeps of 127 rounds of 2 K cycles), 191 us (189 without the
+// residuals).
 __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, float* w, __nv_bfloat16* U, float* evals,
                                                              int r, int eig) {
   extern __shared__ __align__(16) float js[];
@@ -579,9 +582,11 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
       if (evals) evals[h * 128 + 32 * q + lane] = x * unscale;
     }
   }
-  if (tid == 0) atomicMax(reinterpret_cast<int*>(stats + 16), kIter);
+  if (!U || r == 0) {
+    if (tid == 0) atomicMax(reinterpret_cast<int*>(stats + 16), 1);
+    return;
+  }
   __syncthreads();
-  if (!U || r == 0) return;
 
   // ---- LU of T - lambda_j with partial pivoting (lane j of warp 0), pivots of
   // at least 2^-23 in magnitude
@@ -642,8 +647,8 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
     return x;
   };
   float y[16];
-#pragma unroll 1
-  for (int it = 0; it < kIter; ++it) {
+  int it = 0;
+  for (;;) {
     if (warp == 0 && lane < r) {
       // eight steps' operands are loaded before the chain runs through them
       float bc = X[lane];
@@ -694,6 +699,7 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
       }
     }
     __syncthreads();
+    bool bad = false;   // a residual above the tolerance, or no vector left
     // modified Gram-Schmidt, largest eigenvalue first
     if (tid < nact) {
       float mx = 0.0f;
@@ -725,6 +731,7 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
           if (vec == j) {
             const float sc1 = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
             lost |= n2 < 1e-2f * n0;
+            bad |= !(n2 > 0.0f);
 #pragma unroll
             for (int m = 0; m < 16; ++m) y[m] *= sc1;
 #pragma unroll
@@ -752,12 +759,36 @@ __global__ void __launch_bounds__(kBThreads, 1) basis_kernel(uint8_t* stats, flo
           lost = false;
         }
       }
-      if (it + 1 < kIter)
+      // T y - lambda y: the neighbouring entries come from the lanes beside
+      if (it + 1 >= kIter) {
+        const float lam = js[Q_LAM + vec];
 #pragma unroll
-        for (int m = 0; m < 16; ++m) X[(4 * (vp + 8 * (m >> 2)) + (m & 3)) * kXs + vec] = y[m] * 9.5367432e-7f;
+        for (int m = 0; m < 4; ++m) {
+          const int i0 = 4 * (vp + 8 * m), base = lane & 24;
+          const float before = vp == 7 ? (m > 0 ? y[4 * m - 1] : 0.0f) : y[4 * m + 3];
+          const float after = vp == 0 ? (m < 3 ? y[4 * m + 4] : 0.0f) : y[4 * m];
+          const float lf = __shfl_sync(0xFFFFFFFFu, before, base | ((vp + 7) & 7));
+          const float rt = __shfl_sync(0xFFFFFFFFu, after, base | ((vp + 1) & 7));
+          const float4 dv = *reinterpret_cast<const float4*>(js + Q_D + i0);
+          const float4 ev = *reinterpret_cast<const float4*>(js + Q_E + i0);   // e[i] couples i - 1 and i
+          const float e4 = i0 + 4 < 128 ? js[Q_E + i0 + 4] : 0.0f;
+          const float r0 = fmaf(dv.x - lam, y[4 * m], fmaf(ev.x, lf, ev.y * y[4 * m + 1]));
+          const float r1 = fmaf(dv.y - lam, y[4 * m + 1], fmaf(ev.y, y[4 * m], ev.z * y[4 * m + 2]));
+          const float r2 = fmaf(dv.z - lam, y[4 * m + 2], fmaf(ev.z, y[4 * m + 1], ev.w * y[4 * m + 3]));
+          const float r3 = fmaf(dv.w - lam, y[4 * m + 3], fmaf(ev.w, y[4 * m + 2], e4 * rt));
+          bad |= !(fmaxf(fmaxf(fabsf(r0), fabsf(r1)), fmaxf(fabsf(r2), fabsf(r3))) <= kResidual);
+        }
+      }
     }
+    // two steps, and more while a residual is above the tolerance
+    ++it;
+    if (!__syncthreads_or(it < kIter || bad) || it == kMaxIter) break;
+    if (tid < nact)
+#pragma unroll
+      for (int m = 0; m < 16; ++m) X[(4 * (vp + 8 * (m >> 2)) + (m & 3)) * kXs + vec] = y[m] * 9.5367432e-7f;
     __syncthreads();
   }
+  if (tid == 0) atomicMax(reinterpret_cast<int*>(stats + 16), it);
   if (tid >= nact) return;
 
   // ---- back to M's coordinates: H_0 ... H_125 y, two reflections at a time:

@@ -273,3 +273,20 @@ def test_query_basis_is_the_same_without_eigenvalues(H, N, r):
     _, _, lam1 = st.basis(w=False, U=False, eigenvalues=True)
     assert st.read() == (0, N)
     assert torch.equal(w, w1) and torch.equal(U.view(torch.int16), U1.view(torch.int16)) and torch.equal(lam, lam1)
+
+
+def test_query_basis_reports_its_iterations():
+    """sweeps() follows the solver: nothing to iterate for a diagonal matrix or
+    for the eigenvalues alone, the steps until the residuals are small otherwise."""
+    q = workload_queries("single_layer_h4", 0, tokens=880, heads=2).cuda()
+    cfg = qwm.config(2, 64, psac_rank=16)
+    st = qwm.QueryStats(cfg)
+    st.update(torch.eye(128).bfloat16()[:, None].repeat(1, 2, 1).cuda())
+    assert st.sweeps() == 0
+    st.basis(w=True, U=True, eigenvalues=True)
+    assert st.sweeps() == 1
+    st.update(q)
+    st.basis(w=True, U=False, eigenvalues=True)
+    assert st.sweeps() == 1
+    st.basis(w=True, U=True)
+    assert 2 <= st.sweeps() < 30
