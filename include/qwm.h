@@ -270,10 +270,13 @@ QWM_API qwm_status qwm_attend(const qwm_config* cfg, const qwm_cache* cache, con
  * current device; 0 for invalid arguments.  Not part of the paper's method.
  * From 512 keys (1024 in a single chunk) the scratch holds every key and value
  * rebuilt once in binary16 -- 512 bytes per token and head, of as many heads at a
- * time as fit 2 GiB (one at least) -- and up to 41 MB of partial results of query blocks whose keys are split over several CTAs.  With
- * fewer keys, and for calls that want the log-sum-exp, it holds the partial
- * results of the work units of a partly idle last wave (512 queries of one head,
- * split along the keys at whole chunks).  Partial results are combined by the
+ * time as fit 2 GiB (one at least; 671 MB for 40 heads and 32760 keys) -- and up
+ * to 41 MB of partial results of query blocks whose keys are split over several
+ * CTAs.  With fewer keys, and for calls that want the log-sum-exp, it holds the
+ * partial results of the work units of a partly idle last wave (512 queries of
+ * one head, split along the keys at whole chunks; 37 MB at that layer), and a
+ * buffer of that size serves: this call does not know whether the log-sum-exp
+ * will be wanted and gives the larger size.  Partial results are combined by the
  * usual rescaling of partial softmax sums, as for attention over several key
  * blocks. */
 QWM_API size_t qwm_attend_workspace_bytes(const qwm_config* cfg, const qwm_cache* cache, int64_t Nq, int64_t N_cur);
@@ -281,10 +284,13 @@ QWM_API size_t qwm_attend_workspace_bytes(const qwm_config* cfg, const qwm_cache
 /* qwm_attend with a caller-owned device scratch buffer (256-byte aligned) of
  * at least qwm_attend_workspace_bytes bytes for the same arguments: the same
  * result within the attention tolerance (sums in another order; the bf16 output
- * and the lse may differ from qwm_attend's in the last bits; with lse = NULL the
- * PSAC correction is added to the rebuilt keys before their rounding to
- * binary16).  Nothing in the buffer is kept between calls.  workspace = NULL, or
- * a buffer too small, runs qwm_attend.  Calls sharing a buffer must not overlap
+ * and the lse may differ from qwm_attend's in the last bits; with lse = NULL and
+ * from 512 keys the PSAC correction is added to the rebuilt keys before their
+ * rounding to binary16, so out may differ in its last bits between a call that
+ * wants the lse and one that does not).  Nothing in the buffer is kept between
+ * calls.  A buffer too small for the rebuilt keys runs the kernel that rebuilds
+ * them itself, with its partial results where the buffer holds those;
+ * workspace = NULL, or a buffer too small for either, runs qwm_attend.  Calls sharing a buffer must not overlap
  * on the GPU. */
 QWM_API qwm_status qwm_attend_ws(const qwm_config* cfg, const qwm_cache* cache, const void* q, int64_t Nq,
                                  const void* k_cur, const void* v_cur, int64_t N_cur, float sm_scale,

@@ -401,9 +401,11 @@ qwm_status attend_impl(const qwm_config* cfg, const qwm_cache* c, const void* q,
   int units = 0;
   int64_t longest = 0;
   const int64_t Nk = total_keys(c, N_cur, &units, &longest);
-  // The images' path gives no log-sum-exp: that is fp32, and its last digits
-  // follow where the running maximum and the binary16 probabilities are
-  // rounded, which the other kernel's results fix.
+  // The images' path gives no log-sum-exp.  Neither kernel's is nearer the exact
+  // value, but this one's would differ from the other's by 1e-5 to 4e-5 of its
+  // norm (the running maxima, and with them the rounding of the binary16
+  // probabilities, follow the key tiles, which lie elsewhere), and partial
+  // attentions merged by it over several calls should all come from one.
   if (workspace && use_images(units, Nk) && !lse) {
     const DenseGroups g = dense_groups(Nq, c->L.H, Nk, nsm);
     if (workspace_bytes >= g.bytes) {
