@@ -809,6 +809,13 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const DenseArgs a) 
 // log2(e)); a warp per query row, four channels per lane, eight rows of one
 // block per CTA.  A block that one CTA ran over every key is already in the
 // output.
+// Bound by the latency of its loads: B parts' rows are fetched ahead of their
+// sums, the first B ahead of the maximum.  Four at a time without that, 35
+// parts of 128 rows (4 heads, 15 x 880 keys) took 15 us, now 8, the whole call
+// 45 and 35 us (38 in the kernel without images).  B = 8 where a block has more
+// than four parts, else 4: with few parts and many blocks the registers of eight
+// rows cost a wave (1536 CTAs of three parts: 9.3 us with 8, 7.4 with 4).
+template <int B>
 __global__ void __launch_bounds__(256) dense_combine(const DenseArgs a, int grid) {
   const int lane = threadIdx.x & 31;
   const int k = (int)blockIdx.x >> 5, prow = ((int)blockIdx.x & 31) * 8 + (int)(threadIdx.x >> 5);
@@ -828,25 +835,40 @@ __global__ void __launch_bounds__(256) dense_combine(const DenseArgs a, int grid
   auto at = [&](int p) { return p == 0 ? base : (size_t)(2 * (b0 + p)) * 256 + prow; };   // later parts start here
   const float c = a.sm_scale * 1.4426950408889634f;
   const int np = b1 - b0;
-  float m = -INFINITY;
-  for (int p = lane; p < np; p += 32) m = fmaxf(m, a.part_ml[at(p) * 2]);
+  float4 v[B];
+  auto rows = [&](float4 (&x)[B], int p0) {
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      x[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (p0 + i < np) x[i] = *reinterpret_cast<const float4*>(a.part_o + at(p0 + i) * 128 + 4 * lane);
+    }
+  };
+  auto ml_of = [&](int p) {
+    return p < np ? *reinterpret_cast<const float2*>(a.part_ml + at(p) * 2) : make_float2(-INFINITY, 0.0f);
+  };
+  float2 ml = ml_of(lane);
+  rows(v, 0);
+  float m = ml.x;
+#pragma unroll 1
+  for (int p = lane + 32; p < np; p += 32) m = fmaxf(m, ml_of(p).x);
 #pragma unroll
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  float l = 0.0f;
+  float l = 0.0f, wl = 0.0f;
   float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  for (int p0 = 0; p0 < np; p0 += 32) {
-    float wl = 0.0f;
-    if (p0 + lane < np) {
-      const float2 ml = *reinterpret_cast<const float2*>(a.part_ml + at(p0 + lane) * 2);
+#pragma unroll 1
+  for (int p0 = 0; p0 < np; p0 += B) {
+    if ((p0 & 31) == 0) {   // the weights of the next 32 parts, one per lane
+      if (p0 > 0) ml = ml_of(p0 + lane);
       wl = exp2f((ml.x - m) * c);
       l = fmaf(ml.y, wl, l);
     }
-    const int n = min(32, np - p0);
-#pragma unroll 4
-    for (int p = 0; p < n; ++p) {
-      const float wgt = __shfl_sync(0xFFFFFFFFu, wl, p);
-      const float4 v = *reinterpret_cast<const float4*>(a.part_o + at(p0 + p) * 128 + 4 * lane);
-      o.x = fmaf(v.x, wgt, o.x); o.y = fmaf(v.y, wgt, o.y); o.z = fmaf(v.z, wgt, o.z); o.w = fmaf(v.w, wgt, o.w);
+    float4 u[B];
+    rows(u, p0 + B);
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      const float wgt = __shfl_sync(0xFFFFFFFFu, wl, (p0 & 31) + i);   // 0 past the last part
+      o.x = fmaf(v[i].x, wgt, o.x); o.y = fmaf(v[i].y, wgt, o.y); o.z = fmaf(v[i].z, wgt, o.z); o.w = fmaf(v[i].w, wgt, o.w);
+      v[i] = u[i];
     }
   }
 #pragma unroll
@@ -950,7 +972,7 @@ cudaError_t launch_dense(const DenseArgs& a0, const AttendSlots& slots, const De
   lc.gridDim = dim3((unsigned)(p.n_tail * 32));   // 8 rows per CTA
   lc.blockDim = dim3(256);
   lc.dynamicSmemBytes = 0;
-  if ((e = cudaLaunchKernelEx(&lc, dense_combine, a, p.grid)) != cudaSuccess) return e;
+  if ((e = cudaLaunchKernelEx(&lc, p.tail_parts > 4 ? dense_combine<8> : dense_combine<4>, a, p.grid)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

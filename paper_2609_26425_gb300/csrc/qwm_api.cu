@@ -326,10 +326,12 @@ constexpr size_t kDenseImages = (size_t)2 << 30;
 // heads: 27.9 us against 22.5; 600 keys, 300 queries: 30.0 against 32.1), nor
 // over a single chunk below 1024, which the other kernel runs in one launch (880
 // keys and queries, 4 heads: 30.2 against 31.4; 640: 29.4 against 26.0; 4680,
-// 40 heads: 375 against 681).  Above the line both kernels take about 30 us at
-// the smallest sizes: of 260 shapes of 4 to 40 heads and 512 to 4200 keys the
-// images were slower in six, by 1 to 6 % but for one (4 heads, 120 queries, 5
-// x 383 + 120 keys: 28.3 against 24.4), with no size in common.
+// 40 heads: 375 against 681).  Of 840 shapes above the line (1 to 40 heads, 600
+// to 66K keys in 1 to 40 chunks, 1 to 1000 queries, with and without as many
+// active keys) the images were slower in 14, by one to two of their 33 us (two
+// query blocks of a head against the other kernel's one of 512), but for 12
+// heads, 28080 keys and 400 queries (127 against 122), and 1.56 times as fast on
+// average.
 bool use_images(int units, int64_t Nk) { return Nk >= (units >= 2 ? 512 : 1024); }
 
 struct DenseGroups {

@@ -56,6 +56,9 @@ def image_heads(H, Nk):
     (58, [3200, 3200], 4, 16, 1000, 0, (0, 37, 38, 57), (1, "flat", True)),       # after a whole wave
     (81, [20000], 4, 8, 300, 33700, (0, 40, 41, 80), (0, "flat", True)),          # two groups: 41 and 40 heads
     (40, [4680] * 14, 256, 16, 1024, 1024, (0, 18, 39), (1, "parts", False)),     # a long history
+    (4, [880] * 15, 64, 16, 128, 0, (0, 3), (0, "parts", False)),                 # 35 parts of a block
+    (1, [1000] * 40, 16, 8, 130, 0, (0,), (0, "parts", False)),                   # 105 parts
+    (6, [300, 900], 16, 16, 250, 0, (0, 5), (0, "parts", False)),                 # 4 parts
 ])
 def test_images_forms_match_oracle_and_plain(H, chunks, C, r, Nq, Ncur, heads, form):
     nsm = torch.cuda.get_device_properties(0).multi_processor_count
