@@ -21,7 +21,7 @@
 // 32760 keys, 40 heads), whole call: 3.67 ms there, 2.14-2.24 ms here (rebuild
 // 0.18, attention 1.87 ms = 1.67 PFLOP/s of MMA work; the longer figure under
 // the power cap of back-to-back calls); 15 x 880 + 880 keys, 880 queries, 12
-// heads: 154 -> 109 us; 4 heads, 880 queries, 2640 keys: 42 -> 31 us; 1024
+// heads: 154 -> 109 us; 4 heads, 880 queries, 2640 keys: 42 -> 29 us; 1024
 // queries over 66544 keys, 40 heads: 1.62 -> 1.24 ms.
 //
 // The rebuild writes 512 bytes per token and head; its bulk stores alone take

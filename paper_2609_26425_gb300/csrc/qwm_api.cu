@@ -321,17 +321,16 @@ int device_sms() {
 // groups run one after another in the same buffer.
 constexpr size_t kDenseImages = (size_t)2 << 30;
 
-// Whether a call may take the images' path: its three launches take about 28 us
-// at the least, so not over few keys (400 keys in two units, 100 queries, 40
-// heads: 27.9 us against 22.5; 600 keys, 300 queries: 30.0 against 32.1), nor
-// over a single chunk below 1024, which the other kernel runs in one launch (880
-// keys and queries, 4 heads: 30.2 against 31.4; 640: 29.4 against 26.0; 4680,
-// 40 heads: 375 against 681).  Of 840 shapes above the line (1 to 40 heads, 600
-// to 66K keys in 1 to 40 chunks, 1 to 1000 queries, with and without as many
-// active keys) the images were slower in 14, by one to two of their 33 us (two
-// query blocks of a head against the other kernel's one of 512), but for 12
-// heads, 28080 keys and 400 queries (127 against 122), and 1.56 times as fast on
-// average.
+// Whether a call may take the images' path: its three launches cost more than
+// they save over few keys (400 keys in two units, 100 queries, 40 heads: 27.9 us
+// against 22.5; 600 keys, 300 queries: 30.0 against 32.1) and over a single
+// chunk below 1024, which the other kernel runs in one launch (880 keys and
+// queries, 4 heads: 30.2 against 31.4; 640: 29.4 against 26.0; 4680, 40 heads:
+// 375 against 681).  Of 840 shapes above the line (1 to 40 heads, 600 to 66K keys
+// in 1 to 40 chunks, 1 to 1000 queries, with and without as many active keys) the
+// images were slower in 14, by one to two of their 33 us (two query blocks of a
+// head against the other kernel's one of 512), but for 12 heads, 28080 keys and
+// 400 queries (127 against 122), and 1.56 times as fast on average.
 bool use_images(int units, int64_t Nk) { return Nk >= (units >= 2 ? 512 : 1024); }
 
 struct DenseGroups {
